@@ -32,4 +32,10 @@ int eig_work_alloc(EigWork* w, int n, std::vector<void*>* owned);
 template <typename T>
 int launch_eig(RoundPlan* plan, const T* G, EigWork& w, T* S, double* evals, int m, int n, cudaStream_t st);
 
+// The cluster eigensolver (eig_hj.cu) of FP64 Grams up to HJ_MAX64.  n bounds the Gram.
+constexpr int HJ_MAX64 = 256;
+int hj_prepare();
+template <typename T>
+int launch_hj(RoundPlan* plan, const T* G, T* S, double* evals, int m, int n, cudaStream_t st);
+
 }  // namespace tpcg

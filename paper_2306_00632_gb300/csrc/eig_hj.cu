@@ -1,0 +1,787 @@
+// Eigensolver of the mode Grams (Alg. 1 step 3) on a thread-block cluster: pivoted Cholesky G = L L^T, then
+// one-sided (Hestenes) Jacobi on the columns of L.
+//
+//  1. Pivoted Cholesky of G = Z Z^T is the column-pivoted QR of Z^T (L = R^T up to the row order), the
+//     preconditioning step of Drmac and Veselic's one-sided Jacobi SVD, after which few sweeps are needed.  It ends
+//     when what is left cannot matter for this mode's truncation (FP32: 1% of the budget, FP64: 1e-10 of it) or is
+//     rounding noise of the Gram.  The trace of the remainder is energy the truncation discards, and is counted so.
+//  2. Plane rotations from the right make the columns of L orthogonal, L J = U Sigma: the normalised columns are
+//     eigenvectors of G and their squared norms its eigenvalues, and no rotation matrix is accumulated.
+//  3. The columns lie in shared memory in 2 Ce blocks of b, two blocks per CTA of the cluster.  In a round every CTA
+//     rotates all b^2 pairs of one column of each of its blocks, b disjoint pairs at a time (16 lanes to a pair; the
+//     top block's columns stay in registers), then the blocks move by the circle method through distributed shared
+//     memory.  2 Ce - 1 rounds and the pairs inside the blocks make a sweep in which every pair meets once.  The
+//     cluster waits for itself once a round, not once a step.
+//
+// What bounds it: a chain of about rc steps a sweep (5 to 6 sweeps in FP64, 4 in FP32), each a dot product, its
+// reduction, the rotation's parameters and the rotation.  In FP64 the arithmetic: an FP64 instruction of a warp takes
+// its quarter of the SM 64 cycles, dependent or not, so a step costs what one quarter issues (13 + 4 M / 32
+// instructions for one pair).  Hence one pair per quarter, on as many CTAs as the columns fill so; shears with three
+// FMAs an element; everything that only steers the iteration in FP32; and no rotation of pairs far below the budget.
+// Measured, FP64, a Gram of order 120 and full rank: 1.5 ms (16 CTAs), where the two-sided cyclic Jacobi on 8 CTAs that
+// this replaces took 18 ms at order 97; order 32: 0.22 ms against 0.8 ms.
+#include <math.h>
+
+#include <mutex>
+#include <string>
+
+#include <cooperative_groups.h>
+
+#include "common.cuh"
+#include "eig.cuh"
+
+namespace tpcg {
+
+namespace cgx = cooperative_groups;
+
+// A pair is orthogonal once |a_p . a_q| <= tau |a_p| |a_q|.  FP32: the dot product itself resolves about 4e-7 at 128
+// rows.  FP64: at 2e-13 the truncated tensors were up to five times further from the 64-bit ones than at 1e-14, in
+// the same time.  A sweep whose rotations were all below `last` is the last one: the convergence is quadratic, so the next
+// would only meet products near last^2.
+template <typename T>
+__host__ __device__ constexpr T hj_tau() { return sizeof(T) == 8 ? T(1e-14) : T(2e-6); }
+template <typename T>
+__host__ __device__ constexpr T hj_last() { return sizeof(T) == 8 ? T(1e-8) : T(1.5e-3); }
+
+// Shape of a launch: C CTAs, LPP lanes per pair of columns, RPL rows per lane (orders up to LPP RPL), BT pairs a CTA
+// takes at a time before another CTA joins.
+template <typename T_, int C_, int LPP_, int RPL_, int BT_>
+struct HjShape {
+    using T = T_;
+    static constexpr int C = C_, LPP = LPP_, RPL = RPL_, BT = BT_;
+    static constexpr int ROWS = LPP * RPL;
+    static constexpr int BMAX = (ROWS / C + 1) / 2;              // columns of the largest block, pairs at once
+    static constexpr int NT = BMAX * LPP > 128 ? BMAX * LPP : 128;
+    static constexpr int LD = sizeof(T) == 4 && LPP < 32 ? ROWS + LPP : ROWS;   // FP32: a warp's columns on different banks
+    // two sets of two blocks of columns; the Cholesky's own columns lie in the second set
+    static constexpr size_t SMEM = (size_t)4 * BMAX * LD * sizeof(T);
+};
+
+__device__ __forceinline__ double hj_warp_sum(double v) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// An SM issues an FP64 instruction of a warp every 64 cycles and quarter, conversions included, so what only steers
+// the iteration is done in FP32 and conversions by moving bits.
+// v 2^-off as a float (mantissa cut, not rounded; 0 below FP32's range), and a normal float as a double times 2^off
+__device__ __forceinline__ float hj_to_float(double v, int off) {
+    const int hi = __double2hiint(v);
+    const int e = ((hi >> 20) & 0x7ff) - (1023 - 127) - off;
+    const int bits = (hi & 0x80000000) | (e << 23) | ((hi & 0xfffff) << 3) | ((unsigned)__double2loint(v) >> 29);
+    return e > 0 ? __int_as_float(bits) : 0.f;
+}
+__device__ __forceinline__ double hj_to_double(float f, int off = 0) {
+    const unsigned b = __float_as_uint(f);
+    const int hi = (int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + ((unsigned)(1023 - 127 + off) << 20)));
+    return __hiloint2double(hi, (int)(b << 29));
+}
+
+// 1 / sqrt(d) for d in FP32's normal range: an FP32 estimate and one third-order correction (relative error a few ulp)
+__device__ __forceinline__ double hj_rsqrt(double d) {
+    const double y = hj_to_double(rsqrtf(hj_to_float(d, 0)));
+    const double e = fma(-(d * y), y, 1.0);
+    return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+
+// One pair: x and y are this lane's rows of the two columns (zero for an idle group), ax and ay their squared norms.
+// Whole warps call it.  A pair with |x . y| above tau |x| |y| is rotated: u = tan(theta / 2), s = sin(theta), applied
+// as the shears x -= u y, y += s x, x -= u y (three FMAs an element).  The angle needs no more than FP32: an error of
+// 1e-6 in it leaves 1e-6 of the product for the next sweep; s = 2 u / (1 + u^2) has the working precision, so that the
+// shears make an orthogonal matrix.
+template <typename T, int LPP, int RPL>
+__device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, int rpl, T skip, T floor_g, int& big) {
+    T g = T(0);
+#pragma unroll
+    for (int q = 0; q < RPL; ++q)
+        if (q < rpl) g = fma(x[q], y[q], g);
+#pragma unroll
+    for (int o = LPP / 2; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+    float fa, fb, fg, fd;   // |x|^2, |y|^2, x . y, |y|^2 - |x|^2
+    int off = 0;
+    bool on;
+    if constexpr (sizeof(T) == 8) {   // by a power of two near the larger norm: nothing that counts leaves FP32's range
+        const int hx = __double2hiint(ax), hy = __double2hiint(ay), hs = __double2hiint(skip);
+        off = (max(hx, hy) >> 20) - 1023;
+        fa = hj_to_float(ax, off);
+        fb = hj_to_float(ay, off);
+        fg = hj_to_float(g, off);
+        fd = hj_to_float(ay - ax, off);
+        on = hx > hs || hy > hs;      // both far below the budget: all discarded, whatever their products
+    } else {
+        fa = ax;
+        fb = ay;
+        fg = g;
+        fd = ay - ax;
+        on = fabsf(g) > floor_g;
+    }
+    const float ab = fa * fb, ag = fabsf(fg);
+    const float rab = ab > 0.f ? ab * rsqrtf(ab) : 0.f;
+    if (on && ag > (float)hj_tau<T>() * rab) {
+        // t = tan(theta) = sign(d g) 2 |g| / (|d| + sqrt(d^2 + 4 g^2)); u = t / (1 + sqrt(1 + t^2)), its series in t^2
+        // fitted on [0, 1] to 2e-6
+        const float h = fmaf(fd, fd, 4.f * fg * fg);
+        const float t = copysignf(1.f, fd) * __fdividef(2.f * fg, fmaf(h, rsqrtf(h), fabsf(fd)));
+        const float w = t * t;
+        const float u = t * fmaf(w, fmaf(w, fmaf(w, fmaf(w, fmaf(w, -0.00342296f, 0.0151217f), -0.03403639f), 0.06147052f),
+                                 -0.12491905f), 0.49999894f);
+        const float qf = fmaf(u, u, 1.f);
+        T ud, s;
+        if constexpr (sizeof(T) == 8) {
+            ud = hj_to_double(u);
+            const double q = fma(ud, ud, 1.0), r0 = hj_to_double(__fdividef(1.f, qf));
+            const double e = fma(-q, r0, 1.0);
+            s = hj_to_double(2.f * u) * fma(r0, fma(e, e, e), r0);
+        } else {
+            ud = u;
+            s = 2.f * u * __frcp_rn(qf);
+        }
+        if (fabsf(u) > 1e-30f) {
+            if (ag > (float)hj_last<T>() * rab) big = 1;
+#pragma unroll
+            for (int q = 0; q < RPL; ++q)
+                if (q < rpl) {
+                    const T x1 = fma(-ud, y[q], x[q]);
+                    y[q] = fma(s, x1, y[q]);
+                    x[q] = fma(-ud, y[q], x1);
+                }
+            const float tg = t * fg;   // the norms are exact again at the next sweep
+            if constexpr (sizeof(T) == 8) {
+                if (fabsf(tg) > 1e-30f) {
+                    const double v = hj_to_double(tg, off);
+                    ax -= v;
+                    ay += v;
+                }
+            } else {
+                ax -= tg;
+                ay += tg;
+            }
+        }
+    }
+}
+
+// Truncation rule on the decreasingly sorted eigenvalues lam[0..M) (as truncation_rule in eig.cu, sums by one warp).
+// FP64: the smallest s whose discarded (clamped) eigenvalues, the remainder `rem` and, in strict mode, the rounding
+// uncertainty `unc` of each stay within the budget.  FP32: trace minus the kept eigenvalues.  Returns s before the
+// cap, and in *disc a table of the discarded energy by s (M + 1 entries of shared memory).
+template <typename T>
+__device__ int hj_rule(const double* lam, int M, double trace, double rem, double unc, double budget, double* disc) {
+    const int lane = threadIdx.x & 31;
+    const int per = (M + 31) / 32, lo = min(lane * per, M), hi = min(lo + per, M);
+    double own = 0.0;
+    for (int i = lo; i < hi; ++i) own += lam[i] > 0.0 ? lam[i] : 0.0;
+    int cnt = 0;   // FP64: entries that can be discarded; FP32: kept counts that are not enough
+    if (sizeof(T) == 8) {
+        double after = own;   // sum over this lane's and the later lanes' entries
+        for (int o = 1; o < 32; o <<= 1) {
+            const double v = __shfl_down_sync(0xffffffffu, after, o);
+            if (lane + o < 32) after += v;
+        }
+        double t = __shfl_down_sync(0xffffffffu, after, 1);
+        t = (lane < 31 ? t : 0.0) + rem;
+        if (lane == 31) disc[M] = rem;
+        for (int i = hi - 1; i >= lo; --i) {
+            t += lam[i] > 0.0 ? lam[i] : 0.0;
+            disc[i] = t;
+            if (t + unc * (double)(M - i) <= budget) ++cnt;
+        }
+    } else {
+        double before = own;
+        for (int o = 1; o < 32; o <<= 1) {
+            const double v = __shfl_up_sync(0xffffffffu, before, o);
+            if (lane >= o) before += v;
+        }
+        double t = __shfl_up_sync(0xffffffffu, before, 1);
+        t = trace - (lane > 0 ? t : 0.0);
+        for (int i = lo; i < hi; ++i) {   // i kept
+            disc[i] = t > 0.0 ? t : 0.0;
+            if (!(t <= budget)) ++cnt;
+            t -= lam[i];
+        }
+        if (hi == M && (lo < M || M == 0)) disc[M] = t > 0.0 ? t : 0.0;
+    }
+    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    return sizeof(T) == 8 ? M - cnt : cnt;
+}
+
+template <typename SH>
+__global__ void __launch_bounds__(SH::NT, 1)
+    hj_eig_kernel(RoundPlan* plan, const typename SH::T* __restrict__ G, typename SH::T* __restrict__ S, double* evals,
+                  int m, int max_sweeps, double* prof) {
+    using T = typename SH::T;
+    constexpr int C = SH::C, LPP = SH::LPP, RPL = SH::RPL, LD = SH::LD, ROWS = SH::ROWS, BMAX = SH::BMAX, NT = SH::NT;
+    constexpr int NQ = 2 * BMAX;                    // columns of G per CTA (Cholesky)
+    constexpr unsigned FULL = 0xffffffffu;
+    static_assert(NQ <= 32, "one lane per column in the search for the pivot");
+    cgx::cluster_group cluster = cgx::this_cluster();
+    const int crank = (int)cluster.block_rank();
+    RoundPlan& p = *plan;
+    const int M = p.eM, n = p.n;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    extern __shared__ __align__(16) unsigned char hj_raw[];
+    T* cols = reinterpret_cast<T*>(hj_raw);          // [set][block][position] columns, ld LD
+    __shared__ T nrm[2][2][BMAX];                    // squared norms of the columns, moving with them
+    __shared__ T lbuf[2][ROWS];
+    __shared__ int s_key[2][C], s_idx[2][C];         // candidate pivots of every CTA, by parity of the step
+    __shared__ float s_left[2][C];                   // and what is left of the trace on it
+    __shared__ double s_piv[2][C], dg[NQ];           // their values; remaining diagonal of this CTA's columns
+    __shared__ int dg0[NQ];                          // leading bits of what counts as noise there
+    __shared__ float dgf[sizeof(T) == 4 ? ROWS : 1];
+    __shared__ short piv_of[ROWS];
+    __shared__ int s_flags[2][C];
+    __shared__ double s_red[32], s_rem, lam[ROWS], lsort[ROWS], disc[ROWS + 1];
+    __shared__ double s_tr, s_budget, s_bus;
+    __shared__ T s_trs;
+    __shared__ int s_exp;
+    __shared__ short ord[ROWS];
+    __shared__ unsigned char pivoted[ROWS];
+    __shared__ int s_keep, s_nz;
+    if (M <= 0) {
+        if (crank == 0 && tid == 0) {
+            p.s[m] = 0;
+            if (m == 0) { p.norm2 = 0; p.budget = 0; }
+        }
+        return;
+    }
+    // ---- trace, budget, and the power of two that brings the trace near 1 (FP32 products of squared norms would
+    // leave the exponent's range for small tensors)
+    if (warp == 0) {
+        double t = 0.0;
+        for (int i = lane; i < M; i += 32) t += (double)G[i + (long long)i * M];
+        t = hj_warp_sum(t);
+        if (lane == 0) {
+            s_tr = t;
+            // m > 0: the budget of the first mode's kernel; m = 0: every CTA computes it, CTA 0 stores it below
+            const double n2 = p.rr ? p.gtrace : t;
+            const double bu = m == 0 ? fmax(p.eps * p.eps * n2, p.abs2) * (1.0 / 3.0) : p.budget;
+            const int lim = sizeof(T) == 4 ? 120 : 1000;
+            const int k = t > 0.0 ? max(-lim, min(lim, 1023 - ((__double2hiint(t) >> 20) & 0x7ff))) : 0;
+            s_budget = bu;
+            s_exp = k;
+            s_trs = (T)(t * __hiloint2double((1023 + k) << 20, 0));
+            s_bus = bu * __hiloint2double((1023 + k) << 20, 0);
+        }
+    }
+    __syncthreads();
+    const double trace = p.rr ? p.gtrace : s_tr;     // what the rule works with
+    const double budget = s_budget;
+    const double unc = sizeof(T) == 8 && p.strict ? 4.0 * 2.220446049250313e-16 * trace : 0.0;
+    const bool finite = isfinite(s_tr) && isfinite(trace);
+    const int cap = p.cap;
+    // Nothing can be discarded (a strict rule whose budget is below the uncertainty of one eigenvalue) and nothing is
+    // clipped, or there is nothing to decompose (NaN, Inf: kept as it is, so that the scalars built on it show it):
+    // any orthonormal basis serves, and the identity leaves the tensor unchanged.
+    if (!finite || (sizeof(T) == 8 && unc > budget && (cap <= 0 || M <= cap))) {
+        const int s = cap > 0 && M > cap ? cap : M;
+        for (long long e = (long long)crank * NT + tid; e < (long long)M * s; e += (long long)C * NT) {
+            const int i = (int)(e % M), c = (int)(e / M);
+            S[i + (long long)c * n] = (i == c) ? T(1) : T(0);
+        }
+        cluster.sync();   // every CTA has read the plan
+        if (crank == 0 && tid == 0) {
+            if (m == 0) { p.norm2 = trace; p.budget = budget; }
+            p.s[m] = s;
+        }
+        return;
+    }
+    const T sc = sizeof(T) == 8 ? (T)__hiloint2double((1023 + s_exp) << 20, 0) : (T)__int_as_float((127 + s_exp) << 23);
+    const double unscale = __hiloint2double((1023 - s_exp) << 20, 0);
+    const double bus = s_bus;   // the budget on that scale
+    const T tr = s_trs;
+    const int rpl = (M + LPP - 1) / LPP;
+    // ---- 1. pivoted Cholesky; the columns of L pass through S (ld n): how they are spread over the cluster depends on
+    // their number
+    int rc = 0;
+    if constexpr (sizeof(T) == 8) {
+        // The columns of G are spread over the cluster, column j in CTA j mod C, and every step waits for the cluster
+        // once.
+        T* A = cols + 2 * BMAX * LD;
+        const int nq = M > crank ? (M - crank + C - 1) / C : 0;
+        for (int e = tid; e < nq * ROWS; e += NT) {
+            const int q = e / ROWS, i = e % ROWS;
+            A[q * LD + i] = i < M ? G[i + (long long)(crank + C * q) * M] * sc : T(0);
+        }
+        for (int q = tid; q < NQ; q += NT) {
+            const int j = crank + C * q;
+            const T d = j < M ? G[j + (long long)j * M] * sc : T(-1);
+            dg[q] = d;
+            // an entry below 8 u of what the Gram had there is rounding noise and no candidate
+            dg0[q] = __double2hiint(fmax(8 * 1.1102230246251565e-16 * d, 1e-30));
+        }
+        constexpr int RT = (ROWS + NT - 1) / NT;   // rows of a thread
+        bool alive[RT];
+#pragma unroll
+        for (int a = 0; a < RT; ++a) alive[a] = tid + a * NT < M;
+        cluster.sync();   // everybody is in place: remote writes may begin
+        const float stop_rem = (float)(1e-10 * bus);
+        for (int k = 0; k < M; ++k) {
+            const int par = k & 1;
+            if (warp == 0) {
+                // this CTA's candidate: the largest remaining diagonal entry by its leading bits (ties: the first)
+                const double d = lane < NQ ? dg[lane] : -1.0;
+                const int hi = __double2hiint(d);
+                const int key = lane < NQ && hi > dg0[lane] ? hi : -1;
+                const int best = __reduce_max_sync(FULL, key);
+                const int who = __ffs(__ballot_sync(FULL, key == best)) - 1;
+                float left = hi > 0 ? hj_to_float(d, 0) : 0.f;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) left += __shfl_xor_sync(FULL, left, o);
+                const double dm = __shfl_sync(FULL, d, who);
+                if (lane < C) {
+                    cluster.map_shared_rank(&s_key[par][0], lane)[crank] = best;
+                    cluster.map_shared_rank(&s_idx[par][0], lane)[crank] = who;
+                    cluster.map_shared_rank(&s_left[par][0], lane)[crank] = left;
+                    cluster.map_shared_rank(&s_piv[par][0], lane)[crank] = dm;
+                }
+            }
+            cluster.sync();
+            int best = -1, own = 0;
+            float left = 0.f;
+#pragma unroll
+            for (int r = 0; r < C; ++r) {
+                left += s_left[par][r];
+                if (s_key[par][r] > best) { best = s_key[par][r]; own = r; }
+            }
+            if (best < 0 || !(left > stop_rem)) break;   // the same in every thread of the cluster
+            const int q0 = s_idx[par][own], piv = own + C * q0;
+            // l = A[:, piv] / sqrt(d): the owner leaves the column alone from here on, so it is read where it lies
+            const T* src = cluster.map_shared_rank(A, own) + q0 * LD;
+            T col[RT];
+#pragma unroll
+            for (int a = 0; a < RT; ++a) col[a] = alive[a] ? src[tid + a * NT] : T(0);
+            const T inv = hj_rsqrt(s_piv[par][own]);
+            T* lk = lbuf[par];
+            T* out = k % C == crank ? S + (long long)k * n : nullptr;
+#pragma unroll
+            for (int a = 0; a < RT; ++a) {
+                const int i = tid + a * NT;
+                if (i < ROWS) {
+                    const T l = alive[a] ? col[a] * inv : T(0);
+                    lk[i] = l;
+                    if (out && i < M) out[i] = l;
+                }
+                if (i == piv) alive[a] = false;
+            }
+            if (tid == 0) piv_of[k] = (short)piv;
+            __syncthreads();
+            for (int e = tid; e < nq * ROWS; e += NT) {   // a warp works on one column
+                const int q = e / ROWS, i = e % ROWS;
+                const int j = crank + C * q;
+                const T lj = lk[j];
+                if (i >= M || lj == T(0) || j == piv) continue;   // l is zero on the rows of earlier pivots
+                const T v = fma(-lk[i], lj, A[q * LD + i]);
+                A[q * LD + i] = v;
+                if (i == j) dg[q] = v;
+            }
+            if (own == crank && tid == 0) dg[q0] = T(-1);
+            __syncthreads();
+            rc = k + 1;
+        }
+        // energy outside the columns of L
+        if (warp == 0) {
+            const double d = lane < NQ && dg[lane] > T(0) ? (double)dg[lane] : 0.0;
+            const double t = hj_warp_sum(d);
+            if (lane == 0) cluster.map_shared_rank(&s_red[0], 0)[crank] = t;
+        }
+        cluster.sync();   // columns complete, remote reads done
+        if (crank == 0 && tid == 0) {
+            double t = 0.0;
+            for (int r = 0; r < C; ++r) t += s_red[r];
+            s_rem = t * unscale;
+        }
+    } else {
+        // FP32 arithmetic is cheaper than the cluster's barrier: every CTA factorises the whole Gram, held in registers
+        // (entry (i, j) with j = warp + NW a, i = lane + 32 b), and keeps its own columns
+        constexpr int NW = NT / 32, NA = ROWS / NW, NB = ROWS / 32;
+        float Ar[NA][NB];
+#pragma unroll
+        for (int a = 0; a < NA; ++a)
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                const int i = lane + 32 * b, j = warp + NW * a;
+                Ar[a][b] = (i < M && j < M) ? G[i + (long long)j * M] * sc : 0.f;
+            }
+        for (int i = tid; i < ROWS; i += NT) dgf[i] = i < M ? G[i + (long long)i * M] * sc : -1.f;
+        __syncthreads();
+        const float thr = 1e-9f * tr;
+        const float stop_rem = fmaxf(thr, 0.01f * (float)bus);
+        for (int k = 0; k < M; ++k) {
+            // the largest remaining diagonal entry (ties: the lowest index) and the remaining trace, in every warp
+            float v = -2.f, sm = 0.f;
+            int bi = 0;
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                const float d = dgf[lane + 32 * b];
+                if (d > v) { v = d; bi = lane + 32 * b; }
+                sm += fmaxf(d, 0.f);
+            }
+            const int key = v > thr ? __float_as_int(v) : -1;
+            const int best = __reduce_max_sync(FULL, key);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sm += __shfl_xor_sync(FULL, sm, o);
+            const int piv = __reduce_min_sync(FULL, key == best ? bi : ROWS);
+            if (best < 0 || !(sm > stop_rem)) break;   // the same decision in every thread and CTA
+            float* lk = lbuf[k & 1];
+            if (warp == piv % NW) {
+                const float r = __fsqrt_rn(__int_as_float(best));
+                const int ap = piv / NW;
+                T* out = k % C == crank ? S + (long long)k * n : nullptr;
+#pragma unroll
+                for (int b = 0; b < NB; ++b) {
+                    float a = 0.f;
+#pragma unroll
+                    for (int q = 0; q < NA; ++q) a = (q == ap) ? Ar[q][b] : a;
+                    const int i = lane + 32 * b;
+                    a = (i == piv) ? r : __fdiv_rn(a, r);
+                    lk[i] = a;
+                    if (out && i < M) out[i] = a;
+                }
+            }
+            __syncthreads();
+            float li[NB];
+#pragma unroll
+            for (int b = 0; b < NB; ++b) li[b] = lk[lane + 32 * b];
+#pragma unroll
+            for (int a = 0; a < NA; ++a) {
+                const int j = warp + NW * a;
+                const float lj = lk[j];
+#pragma unroll
+                for (int b = 0; b < NB; ++b) {
+                    const int i = lane + 32 * b;
+                    const float w = (i == piv || j == piv) ? 0.f : fmaf(-li[b], lj, Ar[a][b]);
+                    Ar[a][b] = w;
+                    if (i == j && i < M) dgf[i] = (i == piv || dgf[i] < 0.f) ? -1.f : w;
+                }
+            }
+            __syncthreads();
+            rc = k + 1;
+        }
+        cluster.sync();   // columns complete; everybody is in place: remote writes may begin
+    }
+    // ---- 2. one-sided Jacobi
+    // Ce CTAs of the cluster take part, as few as give every CTA BT pairs at a time: column k is in CTA k mod Ce, block
+    // (k / Ce) & 1, position k / (2 Ce).  The others only wait with the cluster.
+    const int Ce = max(1, min(C, (rc + 2 * SH::BT - 1) / (2 * SH::BT)));
+    const int b = crank < Ce ? max(1, ((rc + Ce - 1) / Ce + 1) / 2) : 0;
+    const int grp = tid / LPP, gl = tid % LPP;
+    for (int e = tid; e < 2 * b * ROWS; e += NT) {
+        const int i = e % ROWS, slot = e / ROWS, k = slot * Ce + crank;
+        cols[((slot & 1) * BMAX + (slot >> 1)) * LD + i] = k < rc && i < M ? S[i + (long long)k * n] : T(0);
+    }
+    __syncthreads();
+    const T skip = sizeof(T) == 8 && !p.strict ? (T)(1e-3 * bus * (double)__fdividef(1.f, (float)M)) : T(0);
+    // (a direction of discarded energy below budget / (M + 1) in all is discarded with any basis of it)
+    const T floor_g = sizeof(T) == 8 ? T(0) : T(1e-12f) * tr;   // FP32 products below this are noise of the factor
+    auto column = [&](int set, int blk, int pos) -> T* { return cols + ((set * 2 + blk) * BMAX + pos) * LD; };
+    int set = 0, nsweeps = 0;
+    T x[RPL], y[RPL];
+    for (int sweep = 0; sweep < max_sweeps && rc > 1; ++sweep) {
+        ++nsweeps;
+        int big = 0;   // a rotation that is not small
+        for (int blk = 0; blk < 2; ++blk) {   // exact squared norms
+            T s = T(0);
+            if (grp < b) {
+                const T* a = column(set, blk, grp);
+#pragma unroll
+                for (int q = 0; q < RPL; ++q)
+                    if (q < rpl) { const T v = a[gl + LPP * q]; s = fma(v, v, s); }
+            }
+#pragma unroll
+            for (int o = LPP / 2; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
+            if (grp < b && gl == 0) nrm[set][blk][grp] = s;
+        }
+        __syncthreads();
+        // pairs inside the two blocks (round robin on b rounded up to even players)
+        const int be = (b + 1) & ~1;
+        for (int step = 0; step < be - 1; ++step) {
+            const int half = be / 2;
+            const int blk = grp / half, k = grp - blk * half;
+            int i = -1, j = -1;
+            if (blk < 2) {
+                const int P = be - 1;
+                if (k == 0) { i = P; j = step; }
+                else {
+                    i = step + k; if (i >= P) i -= P;
+                    j = step - k; if (j < 0) j += P;
+                }
+                if (i > j) { const int t = i; i = j; j = t; }
+                if (j >= b) i = -1;
+            }
+            const bool on = i >= 0;
+            if (__any_sync(FULL, on)) {
+                T* xp = column(set, on ? blk : 0, on ? i : 0) + gl;
+                T* yp = column(set, on ? blk : 0, on ? j : 0) + gl;
+                T ax = on ? nrm[set][blk][i] : T(0), ay = on ? nrm[set][blk][j] : T(0);
+#pragma unroll
+                for (int q = 0; q < RPL; ++q)
+                    if (q < rpl) { x[q] = on ? xp[LPP * q] : T(0); y[q] = on ? yp[LPP * q] : T(0); }
+                hj_pair<T, LPP, RPL>(x, y, ax, ay, rpl, skip, floor_g, big);
+                if (on) {
+#pragma unroll
+                    for (int q = 0; q < RPL; ++q)
+                        if (q < rpl) { xp[LPP * q] = x[q]; yp[LPP * q] = y[q]; }
+                    if (gl == 0) { nrm[set][blk][i] = ax; nrm[set][blk][j] = ay; }
+                }
+            }
+            __syncthreads();
+        }
+        for (int round = 0; round < 2 * Ce - 1; ++round) {
+            const bool act = grp < b;
+            const bool wact = warp * (32 / LPP) < b;   // this warp has a pair (b is 0 where the CTA has none)
+            T ax = T(0);
+            if (wact) {
+                const T* xp = column(set, 0, act ? grp : 0) + gl;
+                ax = act ? nrm[set][0][grp] : T(0);
+#pragma unroll
+                for (int q = 0; q < RPL; ++q)
+                    if (q < rpl) x[q] = act ? xp[LPP * q] : T(0);
+            }
+            for (int k = 0; k < b; ++k) {
+                if (wact) {
+                    int j = grp + k; if (j >= b) j -= b;
+                    T* yp = column(set, 1, act ? j : 0) + gl;
+                    T ay = act ? nrm[set][1][j] : T(0);
+#pragma unroll
+                    for (int q = 0; q < RPL; ++q)
+                        if (q < rpl) y[q] = act ? yp[LPP * q] : T(0);
+                    hj_pair<T, LPP, RPL>(x, y, ax, ay, rpl, skip, floor_g, big);
+                    if (act) {
+#pragma unroll
+                        for (int q = 0; q < RPL; ++q)
+                            if (q < rpl) yp[LPP * q] = y[q];
+                        if (gl == 0) nrm[set][1][j] = ay;
+                    }
+                }
+                __syncthreads();
+            }
+            if (round == 2 * Ce - 2) {   // did this sweep rotate by more than a little? told to every CTA
+                const int any = __syncthreads_or(big);
+                if (tid < C && crank < Ce) cluster.map_shared_rank(&s_flags[sweep & 1][0], tid)[crank] = any;
+            }
+            if (Ce == 1) {
+                if (act) {
+                    T* xp = column(set, 0, grp) + gl;
+#pragma unroll
+                    for (int q = 0; q < RPL; ++q)
+                        if (q < rpl) xp[LPP * q] = x[q];
+                    if (gl == 0) nrm[set][0][grp] = ax;
+                }
+                cluster.sync();
+                continue;
+            }
+            // circle method on the 2 Ce blocks: the top blocks move right (the first stays), the bottom blocks left
+            const int ns = set ^ 1;
+            const int tc = crank == 0 ? 0 : (crank == Ce - 1 ? Ce - 1 : crank + 1);
+            const int tb = crank == 0 ? 0 : (crank == Ce - 1 ? 1 : 0);
+            const int bc = crank == 0 ? 1 : crank - 1, bb = crank == 0 ? 0 : 1;
+            if (act) {
+                T* dst = cluster.map_shared_rank(cols, tc) + ((ns * 2 + tb) * BMAX + grp) * LD + gl;
+#pragma unroll
+                for (int q = 0; q < RPL; ++q)
+                    if (q < rpl) dst[LPP * q] = x[q];
+                if (gl == 0) {
+                    cluster.map_shared_rank(&nrm[0][0][0], tc)[(ns * 2 + tb) * BMAX + grp] = ax;
+                    cluster.map_shared_rank(&nrm[0][0][0], bc)[(ns * 2 + bb) * BMAX + grp] = nrm[set][1][grp];
+                }
+                T* dsb = cluster.map_shared_rank(cols, bc) + ((ns * 2 + bb) * BMAX + grp) * LD + gl;
+                const T* yb = column(set, 1, grp) + gl;
+#pragma unroll
+                for (int q = 0; q < RPL; ++q)
+                    if (q < rpl) dsb[LPP * q] = yb[LPP * q];
+            }
+            cluster.sync();
+            set = ns;
+        }
+        int fl = 0;
+        for (int r = 0; r < Ce; ++r) fl |= s_flags[sweep & 1][r];
+        if (!fl) break;   // no rotation, or only small ones
+    }
+    // ---- 3. eigenvalues (exact squared norms) to CTA 0, decreasing order, truncation rule, normalised kept columns.
+    // 2 Ce - 1 moves bring every block home, so player k is where the Cholesky put it.
+    for (int blk = 0; blk < 2; ++blk) {
+        T s = T(0);
+        if (grp < b) {
+            const T* a = column(set, blk, grp);
+#pragma unroll
+            for (int q = 0; q < RPL; ++q)
+                if (q < rpl) { const T v = a[gl + LPP * q]; s = fma(v, v, s); }
+        }
+#pragma unroll
+        for (int o = LPP / 2; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
+        const int k = (2 * grp + blk) * Ce + crank;
+        if (grp < b && gl == 0 && k < rc)
+            for (int r = 0; r < C; ++r) cluster.map_shared_rank(lam, r)[k] = (double)s;
+    }
+    cluster.sync();
+    for (int i = tid; i < M; i += NT) {   // squared norms are not negative: their bits order as integers
+        if (i < rc) {
+            const double v = lam[i];
+            const long long li = v == v ? __double_as_longlong(v) : -1;
+            int rk = 0;
+            for (int j = 0; j < rc; ++j) {
+                const double w = lam[j];
+                const long long lj = w == w ? __double_as_longlong(w) : -1;
+                rk += (lj > li || (lj == li && j < i)) ? 1 : 0;
+            }
+            ord[i] = (short)rk;
+            lsort[rk] = v * unscale;
+        } else {
+            lsort[i] = 0.0;
+        }
+    }
+    __syncthreads();
+    if (crank == 0) {
+        if (warp == 0) {
+            double rem = s_rem;
+            int nz = 0;
+            if (sizeof(T) == 8 && p.rr) {   // energy outside the Rayleigh-Ritz subspace
+                double all = 0.0;
+                for (int i = lane; i < M; i += 32) all += lsort[i];
+                all = hj_warp_sum(all);
+                rem = fmax(trace - all, 0.0);
+            }
+            for (int i = lane; i < M; i += 32) nz += lsort[i] > 0.0 ? 1 : 0;
+            for (int o = 16; o > 0; o >>= 1) nz += __shfl_xor_sync(FULL, nz, o);
+            int s = hj_rule<T>(lsort, M, trace, rem, unc, budget, disc);
+            __syncwarp();
+            if (lane == 0) {
+                if (s == 0 && trace > 0.0 && (m == 0 ? trace : p.norm2) > 0.0) s = 1;
+                if (cap > 0 && s > cap) s = cap;
+                // a zero column is no direction of the tensor; only the strict rule keeps such (completed below)
+                if (!(sizeof(T) == 8 && p.strict) && s > nz) s = nz;
+                if (m == 0) { p.norm2 = trace; p.budget = budget; }
+                p.s[m] = s;
+                p.discarded += disc[s];
+                s_keep = s;
+                s_nz = nz;
+                if (prof) {   // algorithmic work: the dense symmetric eigen-decomposition count 9 M^3; Gram in, S out
+                    prof[2 * PK_EIG] += 9.0 * (double)M * M * M;
+                    prof[2 * PK_EIG + 1] += (double)sizeof(T) * ((double)M * M + (double)M * s);
+                    prof[2 * PK_SWEEPS] += nsweeps;
+                    prof[2 * PK_SWEEPS + 1] += 1.0;
+                }
+            }
+            __syncwarp();
+            if (lane < C && lane > 0) cluster.map_shared_rank(&s_keep, lane)[0] = s_keep;
+        }
+        for (int i = tid; i < M; i += NT) evals[i] = lsort[i];
+    }
+    cluster.sync();
+    const int s = s_keep;
+    for (int blk = 0; blk < 2; ++blk) {
+        const int k = (2 * grp + blk) * Ce + crank;
+        if (grp < b && k < rc && ord[k] < s && lam[k] > 0.0) {
+            const T inv = lam[k] > 1e-30 ? (T)hj_rsqrt(lam[k]) : (T)(1.0 / sqrt(lam[k]));
+            const T* a = column(set, blk, grp);
+            for (int i = gl; i < M; i += LPP) S[i + (long long)ord[k] * n] = a[i] * inv;
+        }
+    }
+    if constexpr (sizeof(T) == 8) {
+        // The strict rule keeps directions the Gram cannot tell from zero: the basis is completed by unit vectors of
+        // rows the Cholesky did not pivot on, orthogonalised twice against what is there (one CTA; rare).
+        __syncthreads();
+        cluster.sync();
+        if (crank == 0 && s > s_nz) {
+            double* v = reinterpret_cast<double*>(cols);
+            double* w = v + ROWS;
+            int c = s_nz;
+            for (int i = tid; i < M; i += NT) pivoted[i] = 0;
+            __syncthreads();
+            for (int k = tid; k < rc; k += NT) pivoted[piv_of[k]] = 1;
+            __syncthreads();
+            for (int j = 0; j < M && c < s; ++j) {
+                if (pivoted[j] && s_nz == rc) continue;   // the same in every thread
+                for (int i = tid; i < M; i += NT) v[i] = i == j ? 1.0 : 0.0;
+                __syncthreads();
+                for (int pass = 0; pass < 2; ++pass) {
+                    for (int q = warp; q < c; q += NT / 32) {
+                        double d = 0.0;
+                        for (int i = lane; i < M; i += 32) d = fma(S[i + (long long)q * n], v[i], d);
+                        d = hj_warp_sum(d);
+                        if (lane == 0) w[q] = d;
+                    }
+                    __syncthreads();
+                    for (int i = tid; i < M; i += NT) {
+                        double a = v[i];
+                        for (int q = 0; q < c; ++q) a = fma(-w[q], S[i + (long long)q * n], a);
+                        v[i] = a;
+                    }
+                    __syncthreads();
+                }
+                double nn = 0.0;
+                for (int i = lane; i < M; i += 32) nn = fma(v[i], v[i], nn);
+                nn = hj_warp_sum(nn);   // every warp: the same sum
+                if (nn > 1e-12) {
+                    const double inv = 1.0 / sqrt(nn);
+                    for (int i = tid; i < M; i += NT) S[i + (long long)c * n] = v[i] * inv;
+                    ++c;
+                }
+                __syncthreads();
+            }
+            if (c < s && tid == 0) p.s[m] = c;
+        }
+    }
+}
+
+namespace {
+template <typename SH>
+int hj_prepare_one() {
+    TPCG_CUDA(cudaFuncSetAttribute(hj_eig_kernel<SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::SMEM));
+    if (SH::C > 8) TPCG_CUDA(cudaFuncSetAttribute(hj_eig_kernel<SH>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    return TPCG_OK;
+}
+
+template <typename SH>
+int hj_launch_one(RoundPlan* plan, const typename SH::T* G, typename SH::T* S, double* evals, int m, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(SH::C);
+    cfg.blockDim = dim3(SH::NT);
+    cfg.dynamicSmemBytes = SH::SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = SH::C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    TPCG_CUDA(cudaLaunchKernelEx(&cfg, hj_eig_kernel<SH>, plan, G, S, evals, m, 30, prof_dev()));
+    TPCG_CHECK_LAUNCH();
+    return TPCG_OK;
+}
+
+// One pair of columns for each quarter of an SM, by the largest order.  More CTAs for the same columns lose to the
+// cluster's barriers (order 32 of 128 possible: 222 us on four, 323 us on sixteen), fewer to the FP64 pipes (order 120:
+// 1.5 ms on sixteen, 2.0 ms on eight).
+using Hj64a = HjShape<double, 4, 32, 1, 4>;
+using Hj64b = HjShape<double, 8, 32, 2, 4>;
+using Hj64c = HjShape<double, 16, 32, 4, 4>;
+using Hj64d = HjShape<double, 16, 32, 8, 8>;
+}  // namespace
+
+int hj_prepare() {   // once per device: takes driver locks, so it stays off the launch path
+    static std::mutex mu;
+    static bool done[64] = {};
+    int dev = 0;
+    TPCG_CUDA(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) dev = 63;
+    std::lock_guard<std::mutex> lock(mu);
+    if (done[dev]) return TPCG_OK;
+    TPCG_TRY(hj_prepare_one<Hj64a>());
+    TPCG_TRY(hj_prepare_one<Hj64b>());
+    TPCG_TRY(hj_prepare_one<Hj64c>());
+    TPCG_TRY(hj_prepare_one<Hj64d>());
+    done[dev] = true;
+    return TPCG_OK;
+}
+
+template <typename T>
+int launch_hj(RoundPlan* plan, const T* G, T* S, double* evals, int m, int n, cudaStream_t st) {
+    if (n <= Hj64a::ROWS) return hj_launch_one<Hj64a>(plan, G, S, evals, m, st);
+    if (n <= Hj64b::ROWS) return hj_launch_one<Hj64b>(plan, G, S, evals, m, st);
+    if (n <= Hj64c::ROWS) return hj_launch_one<Hj64c>(plan, G, S, evals, m, st);
+    return hj_launch_one<Hj64d>(plan, G, S, evals, m, st);
+}
+template int launch_hj<double>(RoundPlan*, const double*, double*, double*, int, int, cudaStream_t);
+
+}  // namespace tpcg
