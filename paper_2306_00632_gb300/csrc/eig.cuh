@@ -32,8 +32,8 @@ int eig_work_alloc(EigWork* w, int n, std::vector<void*>* owned);
 template <typename T>
 int launch_eig(RoundPlan* plan, const T* G, EigWork& w, T* S, double* evals, int m, int n, cudaStream_t st);
 
-// The cluster eigensolver (eig_hj.cu) of FP64 Grams up to HJ_MAX64.  n bounds the Gram.
-constexpr int HJ_MAX64 = 256;
+// The cluster eigensolver (eig_hj.cu): FP32 Grams up to HJ_MAX32, FP64 Grams up to HJ_MAX64.  n bounds the Gram.
+constexpr int HJ_MAX32 = 128, HJ_MAX64 = 256;
 int hj_prepare();
 template <typename T>
 int launch_hj(RoundPlan* plan, const T* G, T* S, double* evals, int m, int n, cudaStream_t st);

@@ -19,7 +19,9 @@
 // instructions for one pair).  Hence one pair per quarter, on as many CTAs as the columns fill so; shears with three
 // FMAs an element; everything that only steers the iteration in FP32; and no rotation of pairs far below the budget.
 // Measured, FP64, a Gram of order 120 and full rank: 1.5 ms (16 CTAs), where the two-sided cyclic Jacobi on 8 CTAs that
-// this replaces took 18 ms at order 97; order 32: 0.22 ms against 0.8 ms.
+// this replaces took 18 ms at order 97; order 32: 0.22 ms against 0.8 ms.  FP32, where a step is 0.4 us of latencies: order
+// 120 and full rank 0.29 ms (four CTAs), rank 51 0.13 ms, rank 16 0.04 ms, where a ring of columns in one CTA's registers
+// with a barrier a step took 0.92, 0.19 and 0.06 ms.
 #include <math.h>
 
 #include <mutex>
@@ -39,7 +41,7 @@ namespace cgx = cooperative_groups;
 // the same time.  A sweep whose rotations were all below `last` is the last one: the convergence is quadratic, so the next
 // would only meet products near last^2.
 template <typename T>
-__host__ __device__ constexpr T hj_tau() { return sizeof(T) == 8 ? T(1e-14) : T(2e-6); }
+__host__ __device__ constexpr T hj_tau() { return sizeof(T) == 8 ? T(1e-14) : T(5e-7); }
 template <typename T>
 __host__ __device__ constexpr T hj_last() { return sizeof(T) == 8 ? T(1e-8) : T(1.5e-3); }
 
@@ -750,9 +752,11 @@ int hj_launch_one(RoundPlan* plan, const typename SH::T* G, typename SH::T* S, d
     return TPCG_OK;
 }
 
-// One pair of columns for each quarter of an SM, by the largest order.  More CTAs for the same columns lose to the
-// cluster's barriers (order 32 of 128 possible: 222 us on four, 323 us on sixteen), fewer to the FP64 pipes (order 120:
-// 1.5 ms on sixteen, 2.0 ms on eight).
+// FP32: four CTAs of 16 warps; eight CTAs for the same columns were 14% slower at order 120 and full rank, 8 or 16
+// instead of 12 pairs before another CTA joins within 5%.  FP64: one pair of columns for each quarter of an SM, by the
+// largest order.  More CTAs for the same columns lose to the cluster's barriers (order 32 of 128 possible: 222 us on four,
+// 323 us on sixteen), fewer to the FP64 pipes (order 120: 1.5 ms on sixteen, 2.0 ms on eight).
+using Hj32 = HjShape<float, 4, 32, 4, 12>;
 using Hj64a = HjShape<double, 4, 32, 1, 4>;
 using Hj64b = HjShape<double, 8, 32, 2, 4>;
 using Hj64c = HjShape<double, 16, 32, 4, 4>;
@@ -767,6 +771,7 @@ int hj_prepare() {   // once per device: takes driver locks, so it stays off the
     if (dev < 0 || dev >= 64) dev = 63;
     std::lock_guard<std::mutex> lock(mu);
     if (done[dev]) return TPCG_OK;
+    TPCG_TRY(hj_prepare_one<Hj32>());
     TPCG_TRY(hj_prepare_one<Hj64a>());
     TPCG_TRY(hj_prepare_one<Hj64b>());
     TPCG_TRY(hj_prepare_one<Hj64c>());
@@ -777,11 +782,16 @@ int hj_prepare() {   // once per device: takes driver locks, so it stays off the
 
 template <typename T>
 int launch_hj(RoundPlan* plan, const T* G, T* S, double* evals, int m, int n, cudaStream_t st) {
-    if (n <= Hj64a::ROWS) return hj_launch_one<Hj64a>(plan, G, S, evals, m, st);
-    if (n <= Hj64b::ROWS) return hj_launch_one<Hj64b>(plan, G, S, evals, m, st);
-    if (n <= Hj64c::ROWS) return hj_launch_one<Hj64c>(plan, G, S, evals, m, st);
-    return hj_launch_one<Hj64d>(plan, G, S, evals, m, st);
+    if constexpr (sizeof(T) == 4) {
+        return hj_launch_one<Hj32>(plan, G, S, evals, m, st);
+    } else {
+        if (n <= Hj64a::ROWS) return hj_launch_one<Hj64a>(plan, G, S, evals, m, st);
+        if (n <= Hj64b::ROWS) return hj_launch_one<Hj64b>(plan, G, S, evals, m, st);
+        if (n <= Hj64c::ROWS) return hj_launch_one<Hj64c>(plan, G, S, evals, m, st);
+        return hj_launch_one<Hj64d>(plan, G, S, evals, m, st);
+    }
 }
+template int launch_hj<float>(RoundPlan*, const float*, float*, double*, int, int, cudaStream_t);
 template int launch_hj<double>(RoundPlan*, const double*, double*, double*, int, int, cudaStream_t);
 
 }  // namespace tpcg

@@ -3,7 +3,9 @@ around multiples of the lanes of a pair, of the cluster and of its largest sizes
 
 Bounds.  A Gram of ||Z|| = 1 carries rounding errors of about sqrt(M) u; a kept direction of size sigma moves by that
 over sigma.  The smallest kept sigma is above eps / (2 M), so the truncated tensors agree to about
-2 M^1.5 u / eps; ten times that is allowed, which stays below 1e-7 in FP64 for the eps here."""
+2 M^1.5 u / eps; ten times that is allowed, which stays below 1e-7 in FP64 for the eps here.  In FP32 the kernel works
+on G less a Cholesky remainder of up to a hundredth of the budget eps^2 / 3, which turns a kept direction by at most a
+hundredth of eps; eps / 50 is allowed on the tensor, beside the rounding term."""
 import numpy as np
 import pytest
 
@@ -108,3 +110,22 @@ def test_f64_nan_stays_visible(api):
     ctx = api.Ctx(n, n, n)
     api.tucker_round(ctx, y, 1e-3)
     assert not np.isfinite(float(api.tucker_dot(ctx, y, y)))
+
+
+@pytest.mark.parametrize("n,ranks", [(4, (1, 1, 1)), (6, (2, 3, 6)), (20, (15, 16, 17)), (34, (31, 33, 34)),
+                                     (66, (63, 17, 32)), (97, (97, 20, 20)), (127, (127, 65, 12)),
+                                     (128, (128, 24, 24))])
+def test_f32_edges(api, n, ranks):
+    Y = _tensor(n, ranks, 0.05, seed=n)
+    Y = (Y[0].astype(np.float32).astype(float), [u.astype(np.float32).astype(float) for u in Y[1]])
+    eps = _gap_eps(Y, 0.1)
+    ref = rounding.t_rel(Y, eps)
+    y = api.Tucker.from_numpy(Y[0], Y[1], cap=n, core_cap=n * max(ranks) ** 2, dtype=1)
+    ctx = api.Ctx(n, n, n, dtype=1)
+    api.tucker_round(ctx, y, eps)
+    G, U = y.to_numpy()
+    assert G.shape == ref[0].shape
+    M = max(ranks)
+    assert rel(tucker.full((G, U)), tucker.full(ref)) <= 20 * M ** 1.5 * 2.0 ** -24 / eps + eps / 50
+    for t in range(3):
+        assert np.abs(U[t].T @ U[t] - np.eye(U[t].shape[1])).max() < 1e-5
