@@ -28,9 +28,9 @@ int eig_work_alloc(EigWork* w, int n, std::vector<void*>* owned);
 
 // Eigen-decomposition (Jacobi) of the plan's current Gram G (gM x gM, ld gM), truncation rule of mode m, kept
 // eigenvectors (orthonormal) into S (ld n); plan.s[m], plan.discarded (and for m = 0 plan.norm2/budget)
-// are updated on the device.
+// are updated on the device.  n bounds gM; rr: the context reduces large Grams first (n is then RR_L).
 template <typename T>
-int launch_eig(RoundPlan* plan, const T* G, EigWork& w, T* S, double* evals, int m, int n, cudaStream_t st);
+int launch_eig(RoundPlan* plan, const T* G, EigWork& w, T* S, double* evals, int m, int n, bool rr, cudaStream_t st);
 
 // The cluster eigensolver (eig_hj.cu): FP32 Grams up to HJ_MAX32, FP64 Grams up to HJ_MAX64.  n bounds the Gram.
 constexpr int HJ_MAX32 = 128, HJ_MAX64 = 256;

@@ -656,7 +656,7 @@ int round_stage34(tpcg_ctx c, tucker_t* y, double* info_dev, cudaStream_t st) {
             TPCG_CHECK_LAUNCH();
             TPCG_TRY((launch_gemm<T, true, false>(ga, nullptr, 1, 1, RR_L, RR_L, st)));
         }
-        TPCG_TRY(launch_eig<T>(c->plan, Gm, c->eigw, Sm, c->evals, m, c->rr ? RR_L : n, st));
+        TPCG_TRY(launch_eig<T>(c->plan, Gm, c->eigw, Sm, c->evals, m, c->rr ? RR_L : n, c->rr != 0, st));
         if (c->rr) {   // kept Ritz vectors Q U back into S
             rr_step_kernel<T><<<1, 32, 0, st>>>(c->plan, ga, Gm, rQ, rY, Sm, m, 2);
             TPCG_CHECK_LAUNCH();
