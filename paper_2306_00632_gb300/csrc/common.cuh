@@ -82,7 +82,8 @@ static_assert(sizeof(TuckerDesc) <= TPCG_DESC_BYTES, "descriptor too large");
 // needed: then C = beta*C when K = 0).
 struct GemmArgs {
     int M, N, K, nbatch;
-    int acc, pad0;
+    int acc;
+    int sym;            // the product is symmetric and only the tiles of its lower triangle have to be computed
     const void* A;
     long long lda, sA;
     const void* B;

@@ -14,6 +14,7 @@
 // sequence of launches without synchronising.
 #include <math.h>
 
+#include <algorithm>
 #include <string>
 
 #include "common.cuh"
@@ -262,7 +263,7 @@ __device__ void plan_gram(RoundPlan& p, GemmArgs* ga, const T* Zc, T* Part, int 
         if (hi > total) hi = total;
         if (lo >= hi) break;
         GemmArgs a{};
-        a.M = M; a.N = M; a.alpha = 1.0; a.beta = 0.0;
+        a.M = M; a.N = M; a.alpha = 1.0; a.beta = 0.0; a.sym = 1;
         a.C = Part + (long long)used * M * M; a.ldc = M; a.sC = 0;
         if (m == 0) {
             a.K = hi - lo; a.nbatch = 1; a.acc = 0;
@@ -287,6 +288,24 @@ __device__ void plan_gram(RoundPlan& p, GemmArgs* ga, const T* Zc, T* Part, int 
     counts[0] = used;
     counts[1] = M;
     counts[2] = M;
+}
+
+// G = the sum of the partial Grams in their order, from their lower triangles (the GEMM need not compute the others);
+// M and the number of partials read from the device
+template <typename T>
+__global__ void __launch_bounds__(256) gram_reduce_kernel(const T* __restrict__ P, const int* __restrict__ counts,
+                                                          T* __restrict__ G) {
+    const int cnt = counts[0], M = counts[1];
+    const long long MM = (long long)M * M;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < MM; e += (long long)gridDim.x * blockDim.x) {
+        const int i = (int)(e % M), j = (int)(e / M);
+        if (i < j) continue;
+        T s = T(0);
+#pragma unroll 16
+        for (int g = 0; g < cnt; ++g) s += P[g * MM + e];
+        G[e] = s;
+        G[j + (long long)i * M] = s;
+    }
 }
 
 template <typename T>
@@ -580,7 +599,6 @@ int round_stage12(tpcg_ctx c, tucker_t* y, double eps, const double* eps_dev, in
     GemmArgs* ga = c->gargs;
     int* counts = reinterpret_cast<int*>(c->scal + 200);   // 8 ints of scratch in the scalar area
     T* Z0 = static_cast<T*>(c->Z0);
-    T* Z1 = static_cast<T*>(c->Z1);
     plan_round_kernel<T><<<1, 32, 0, st>>>(static_cast<const TuckerDesc*>(y->desc), c->plan, ga, n, rc, eps, eps_dev,
                                            c->Rq[0], c->Rq[1], c->Rq[2], y->U[0], y->U[1], y->U[2],
                                            static_cast<T*>(c->T1), static_cast<T*>(c->Wm), counts,
@@ -631,11 +649,11 @@ int round_stage34(tpcg_ctx c, tucker_t* y, double* info_dev, cudaStream_t st) {
     for (int m = 0; m < 3; ++m) {
         prof_begin(PK_GRAM, st);
         if (m == 0)
-            TPCG_TRY((launch_gemm<T, false, true>(ga, counts, MAX_SPLIT, 1, n, n, st)));
+            TPCG_TRY((launch_gemm<T, false, true>(ga, counts, MAX_SPLIT, 1, n, n, st, true)));
         else
-            TPCG_TRY((launch_gemm<T, true, false>(ga, counts, MAX_SPLIT, 1, n, n, st)));
-        reduce_partials_kernel<T><<<64, 256, 0, st>>>(static_cast<T*>(c->Part), counts + 1, counts + 2, counts,
-                                                      static_cast<T*>(c->Gm), 0, 1.0, 0.0);
+            TPCG_TRY((launch_gemm<T, true, false>(ga, counts, MAX_SPLIT, 1, n, n, st, true)));
+        gram_reduce_kernel<T><<<std::min((n * n + 255) / 256, 2 * sm_count()), 256, 0, st>>>(
+            static_cast<const T*>(c->Part), counts, static_cast<T*>(c->Gm));
         TPCG_CHECK_LAUNCH();
         prof_end(PK_GRAM, st);
         prof_begin(PK_EIG, st);
