@@ -282,6 +282,7 @@ extern "C" int tpcg_ctx_create(int n, int max_cols, int rank_cap, int dtype, tpc
     TPCG_TRY(eig_prepare());
     TPCG_TRY(tc_prepare());
     TPCG_TRY(gemm32_prepare());
+    TPCG_TRY(qr_prepare());
     (void)sm_count();
     tpcg_ctx c = new tpcg_ctx_s();
     c->lo = nullptr;

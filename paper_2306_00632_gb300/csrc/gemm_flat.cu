@@ -5,7 +5,7 @@
 // and takes tiles blockIdx.x, blockIdx.x + gridDim.x, ... of that list: no CTA walks over empty groups, and the tiles
 // of many small products spread over the chip like those of one large one.  Sums run in the order of k as in the kernels
 // this replaces, so results keep their bits.  Measured, whole truncations: operator product n = 128 (19 blocks of rank 36,
-// FP32) 1.48 -> 1.23 ms, its 19 products with a long side 175 us -> 20 us; n = 512, FP32, 19.9 -> 10.7 ms; n = 97, FP64,
+// FP32) 1.48 -> 1.23 ms, its 19 products with a long side 175 us -> 32 us; n = 512, FP32, 19.9 -> 10.7 ms; n = 97, FP64,
 // 5.3 -> 3.8 ms; a scalar product of rank 6 at n = 32 130 -> 66 us.
 #include <math.h>
 

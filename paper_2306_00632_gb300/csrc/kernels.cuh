@@ -21,6 +21,11 @@ int round_resolved(tpcg_ctx c, const tucker_t* y, tucker_t* out, double eps, con
                    double* norm2_slot, tucker_t* E, tucker_t* F, cudaStream_t st);
 int round_mixed(tpcg_ctx c64, tpcg_ctx c32, tucker_t* y64, tucker_t* out32, double eps, const double* eps_dev, int cap,
                 double abs_tol, double* info_dev, cudaStream_t st);
+// Householder QR Y_t = Q_t R_t of the modes with k_t < n (qr.cu), n <= QR_MAXN; W: n x n working copies, ld n everywhere
+constexpr int QR_MAXN = 512;
+int qr_prepare();
+template <typename T>
+int launch_qr(const RoundPlan* plan, int n, const T* const* Y, T* const* W, T* const* R, T* const* Q, cudaStream_t st);
 // whether a context of this size, rank cap and dtype reduces its large Grams by Rayleigh-Ritz
 int rr_kind();      // TPCG_OPT_RR
 int gram_min_k();   // TPCG_OPT_GRAM_MIN_K

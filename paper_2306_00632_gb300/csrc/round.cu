@@ -1,7 +1,7 @@
 // Relative-tolerance truncation of a Tucker tensor (Alg. 1 with ST-HOSVD), device-driven.
 //
 //   step 1  QR of each factor Y_t (n x k_t).  When k_t >= n any orthonormal Q_t spanning R^n serves, so
-//           Q_t = I and R_t = Y_t (no work); otherwise a Householder QR in one CTA per mode.
+//           Q_t = I and R_t = Y_t (no work); otherwise a Householder QR (qr.cu).
 //   step 2  Z = sum_b scale_b G_b x_1 R_1^(b) x_2 R_2^(b) x_3 R_3^(b) over the core blocks b
 //           (block-diagonal core): per block the middle mode on the small core, then mode 1, writing
 //           the block's slab of a stacked matrix W; one fused GEMM over all blocks contracts mode 3.
@@ -212,7 +212,7 @@ __device__ void householder_qr(const T* Y, T* A, T* R, T* Q, int rows, int k, lo
     }
 }
 
-// Alg. 1 step 1: Y_t = Q_t R_t for the modes with k_t < n, one CTA per mode (n x k_t, ld n)
+// Alg. 1 step 1 above n = QR_MAXN: Y_t = Q_t R_t for the modes with k_t < n, one CTA per mode (n x k_t, ld n)
 template <typename T>
 __global__ void __launch_bounds__(1024) qr_kernel(const RoundPlan* __restrict__ plan, const T* Y0, const T* Y1,
                                                   const T* Y2, T* W0, T* W1, T* W2, T* R0, T* R1, T* R2, T* Q0,
@@ -606,7 +606,17 @@ int round_stage12(tpcg_ctx c, tucker_t* y, double eps, const double* eps_dev, in
     TPCG_CHECK_LAUNCH();
     // step 1: QR where k_t < n
     prof_begin(PK_QR, st);
-    {
+    if (n <= QR_MAXN) {
+        const T* Y[3];
+        T *W[3], *R[3], *Q[3];
+        for (int t = 0; t < 3; ++t) {
+            Y[t] = static_cast<const T*>(y->U[t]);
+            W[t] = static_cast<T*>(c->Yw[t]);
+            R[t] = static_cast<T*>(c->Rq[t]);
+            Q[t] = static_cast<T*>(c->Qq[t]);
+        }
+        TPCG_TRY(launch_qr<T>(c->plan, n, Y, W, R, Q, st));
+    } else {
         size_t sm = (size_t)(n + 40) * sizeof(T);
         qr_kernel<T><<<3, 1024, sm, st>>>(c->plan, static_cast<const T*>(y->U[0]), static_cast<const T*>(y->U[1]),
                                           static_cast<const T*>(y->U[2]), static_cast<T*>(c->Yw[0]),
