@@ -26,6 +26,7 @@
 
 #include <mutex>
 #include <string>
+#include <type_traits>
 
 #include <cooperative_groups.h>
 
@@ -117,47 +118,59 @@ __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, 
         fd = ay - ax;
         on = fabsf(g) > floor_g;
     }
+    // t = tan(theta) = sign(d g) 2 |g| / (|d| + sqrt(d^2 + 4 g^2)); u = t / (1 + sqrt(1 + t^2)), its series in t^2 fitted
+    // on [0, 1] to 2e-6.  Formed beside the test, not after it.
     const float ab = fa * fb, ag = fabsf(fg);
-    const float rab = ab > 0.f ? ab * rsqrtf(ab) : 0.f;
-    if (on && ag > (float)hj_tau<T>() * rab) {
-        // t = tan(theta) = sign(d g) 2 |g| / (|d| + sqrt(d^2 + 4 g^2)); u = t / (1 + sqrt(1 + t^2)), its series in t^2
-        // fitted on [0, 1] to 2e-6
-        const float h = fmaf(fd, fd, 4.f * fg * fg);
-        const float t = copysignf(1.f, fd) * __fdividef(2.f * fg, fmaf(h, rsqrtf(h), fabsf(fd)));
-        const float w = t * t;
-        const float u = t * fmaf(w, fmaf(w, fmaf(w, fmaf(w, fmaf(w, -0.00342296f, 0.0151217f), -0.03403639f), 0.06147052f),
-                                 -0.12491905f), 0.49999894f);
-        const float qf = fmaf(u, u, 1.f);
+    const float h = fmaf(fd, fd, 4.f * fg * fg);
+    const float t = copysignf(1.f, fd) * __fdividef(2.f * fg, fmaf(h, rsqrtf(h), fabsf(fd)));
+    const float w = t * t;
+    const float u = t * fmaf(w, fmaf(w, fmaf(w, fmaf(w, fmaf(w, -0.00342296f, 0.0151217f), -0.03403639f), 0.06147052f),
+                             -0.12491905f), 0.49999894f);
+    bool above, large;
+    if constexpr (sizeof(T) == 8) {
+        const float rab = ab > 0.f ? ab * rsqrtf(ab) : 0.f;
+        above = ag > (float)hj_tau<T>() * rab;
+        large = ag > (float)hj_last<T>() * rab;
+    } else {
+        above = ag * ag > hj_tau<T>() * hj_tau<T>() * ab;
+        large = ag * ag > hj_last<T>() * hj_last<T>() * ab;
+    }
+    if (on && above && fabsf(u) > 1e-30f) {
+        if (large) big = 1;
         T ud, s;
         if constexpr (sizeof(T) == 8) {
             ud = hj_to_double(u);
-            const double q = fma(ud, ud, 1.0), r0 = hj_to_double(__fdividef(1.f, qf));
-            const double e = fma(-q, r0, 1.0);
-            s = hj_to_double(2.f * u) * fma(r0, fma(e, e, e), r0);
+            const double u2 = hj_to_double(2.f * u);
+            if (fabsf(u) < 1e-4f && fabsf(u) > 1e-15f) {   // 2 u (1 - u^2) to u^4
+                s = fma(-u2, hj_to_double(u * u), u2);
+            } else {
+                const float qf = fmaf(u, u, 1.f);
+                const double q = fma(ud, ud, 1.0), r0 = hj_to_double(__fdividef(1.f, qf));
+                const double e = fma(-q, r0, 1.0);
+                s = u2 * fma(r0, fma(e, e, e), r0);
+            }
         } else {
             ud = u;
-            s = 2.f * u * __frcp_rn(qf);
+            const float q = fmaf(u, u, 1.f), r0 = __fdividef(1.f, q);
+            s = 2.f * u * fmaf(r0, fmaf(-q, r0, 1.f), r0);
         }
-        if (fabsf(u) > 1e-30f) {
-            if (ag > (float)hj_last<T>() * rab) big = 1;
 #pragma unroll
-            for (int q = 0; q < RPL; ++q)
-                if (q < rpl) {
-                    const T x1 = fma(-ud, y[q], x[q]);
-                    y[q] = fma(s, x1, y[q]);
-                    x[q] = fma(-ud, y[q], x1);
-                }
-            const float tg = t * fg;   // the norms are exact again at the next sweep
-            if constexpr (sizeof(T) == 8) {
-                if (fabsf(tg) > 1e-30f) {
-                    const double v = hj_to_double(tg, off);
-                    ax -= v;
-                    ay += v;
-                }
-            } else {
-                ax -= tg;
-                ay += tg;
+        for (int q = 0; q < RPL; ++q)
+            if (q < rpl) {
+                const T x1 = fma(-ud, y[q], x[q]);
+                y[q] = fma(s, x1, y[q]);
+                x[q] = fma(-ud, y[q], x1);
             }
+        const float tg = t * fg;   // the norms are exact again at the next sweep
+        if constexpr (sizeof(T) == 8) {
+            if (fabsf(tg) > 1e-30f) {
+                const double v = hj_to_double(tg, off);
+                ax -= v;
+                ay += v;
+            }
+        } else {
+            ax -= tg;
+            ay += tg;
         }
     }
 }
@@ -291,17 +304,25 @@ __global__ void __launch_bounds__(SH::NT, 1)
     const double bus = s_bus;   // the budget on that scale
     const T tr = s_trs;
     const int rpl = (M + LPP - 1) / LPP;
-    // ---- 1. pivoted Cholesky; the columns of L pass through S (ld n): how they are spread over the cluster depends on
-    // their number
+    // ---- 1. pivoted Cholesky.  How the columns of L are spread over the cluster depends on their number: they wait in
+    // shared memory (FP64) or in S (FP32)
     int rc = 0;
     if constexpr (sizeof(T) == 8) {
         // The columns of G are spread over the cluster, column j in CTA j mod C, and every step waits for the cluster
         // once.
-        T* A = cols + 2 * BMAX * LD;
-        const int nq = M > crank ? (M - crank + C - 1) / C : 0;
-        for (int e = tid; e < nq * ROWS; e += NT) {
-            const int q = e / ROWS, i = e % ROWS;
-            A[q * LD + i] = i < M ? G[i + (long long)(crank + C * q) * M] * sc : T(0);
+        T* A = cols + 2 * BMAX * LD;                     // what other CTAs read; the own columns are in registers as well
+        constexpr int RT = (ROWS + NT - 1) / NT, CT = RT == 1 && NT > ROWS ? NT / ROWS : 1, QT = (NQ + CT - 1) / CT;
+        const int row = CT > 1 ? tid % ROWS : tid, cg = CT > 1 ? tid / ROWS : 0;   // rows row + NT a, columns cg + CT q
+        double Ar[RT][QT];
+#pragma unroll
+        for (int q = 0; q < QT; ++q) {
+            const int cq = cg + CT * q, j = crank + C * cq;
+#pragma unroll
+            for (int a = 0; a < RT; ++a) {
+                const int i = row + NT * a;
+                Ar[a][q] = i < M && j < M ? G[i + (long long)j * M] * sc : T(0);
+                if (cq < NQ && i < ROWS) A[cq * LD + i] = Ar[a][q];
+            }
         }
         for (int q = tid; q < NQ; q += NT) {
             const int j = crank + C * q;
@@ -310,10 +331,9 @@ __global__ void __launch_bounds__(SH::NT, 1)
             // an entry below 8 u of what the Gram had there is rounding noise and no candidate
             dg0[q] = __double2hiint(fmax(8 * 1.1102230246251565e-16 * d, 1e-30));
         }
-        constexpr int RT = (ROWS + NT - 1) / NT;   // rows of a thread
         bool alive[RT];
 #pragma unroll
-        for (int a = 0; a < RT; ++a) alive[a] = tid + a * NT < M;
+        for (int a = 0; a < RT; ++a) alive[a] = row + NT * a < M;
         cluster.sync();   // everybody is in place: remote writes may begin
         const float stop_rem = (float)(1e-10 * bus);
         for (int k = 0; k < M; ++k) {
@@ -325,55 +345,68 @@ __global__ void __launch_bounds__(SH::NT, 1)
                 const int key = lane < NQ && hi > dg0[lane] ? hi : -1;
                 const int best = __reduce_max_sync(FULL, key);
                 const int who = __ffs(__ballot_sync(FULL, key == best)) - 1;
-                float left = hi > 0 ? hj_to_float(d, 0) : 0.f;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) left += __shfl_xor_sync(FULL, left, o);
                 const double dm = __shfl_sync(FULL, d, who);
                 if (lane < C) {
                     cluster.map_shared_rank(&s_key[par][0], lane)[crank] = best;
                     cluster.map_shared_rank(&s_idx[par][0], lane)[crank] = who;
-                    cluster.map_shared_rank(&s_left[par][0], lane)[crank] = left;
                     cluster.map_shared_rank(&s_piv[par][0], lane)[crank] = dm;
                 }
+            } else if (warp == 1) {   // what is left of the trace
+                const double d = lane < NQ ? dg[lane] : -1.0;
+                float left = __double2hiint(d) > 0 ? hj_to_float(d, 0) : 0.f;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) left += __shfl_xor_sync(FULL, left, o);
+                if (lane < C) cluster.map_shared_rank(&s_left[par][0], lane)[crank] = left;
             }
             cluster.sync();
-            int best = -1, own = 0;
-            float left = 0.f;
+            const int ky = lane < C ? s_key[par][lane] : -1;
+            float left = lane < C ? s_left[par][lane] : 0.f;
+            const int best = __reduce_max_sync(FULL, ky);
+            const int own = __ffs(__ballot_sync(FULL, ky == best)) - 1;
 #pragma unroll
-            for (int r = 0; r < C; ++r) {
-                left += s_left[par][r];
-                if (s_key[par][r] > best) { best = s_key[par][r]; own = r; }
-            }
+            for (int o = 8; o > 0; o >>= 1) left += __shfl_xor_sync(FULL, left, o);
+            left = __shfl_sync(FULL, left, 0);
             if (best < 0 || !(left > stop_rem)) break;   // the same in every thread of the cluster
             const int q0 = s_idx[par][own], piv = own + C * q0;
-            // l = A[:, piv] / sqrt(d): the owner leaves the column alone from here on, so it is read where it lies
+            // Column a = A[:, piv] as it is, and 1 / d: A -= a a^T / d.  The scaling of L's column waits until it is read
+            // back.  The owner leaves the column alone from here on, so it is read where it lies.
             const T* src = cluster.map_shared_rank(A, own) + q0 * LD;
             T col[RT];
 #pragma unroll
-            for (int a = 0; a < RT; ++a) col[a] = alive[a] ? src[tid + a * NT] : T(0);
-            const T inv = hj_rsqrt(s_piv[par][own]);
+            for (int a = 0; a < RT; ++a) col[a] = alive[a] ? src[row + a * NT] : T(0);
+            const double d = s_piv[par][own];
+            const double r0 = hj_to_double(__fdividef(1.f, hj_to_float(d, 0)));
+            const double er = fma(-d, r0, 1.0), invd = fma(r0, fma(er, er, er), r0);
             T* lk = lbuf[par];
-            T* out = k % C == crank ? S + (long long)k * n : nullptr;
+            T* out = k % C == crank ? cols + (k / C) * LD : nullptr;   // (a store to global memory here makes the barrier wait)
 #pragma unroll
             for (int a = 0; a < RT; ++a) {
-                const int i = tid + a * NT;
-                if (i < ROWS) {
-                    const T l = alive[a] ? col[a] * inv : T(0);
-                    lk[i] = l;
-                    if (out && i < M) out[i] = l;
+                const int i = row + a * NT;
+                if (cg == 0 && i < ROWS) {
+                    lk[i] = col[a];
+                    if (out) out[i] = col[a];
                 }
                 if (i == piv) alive[a] = false;
+                col[a] *= -invd;
             }
-            if (tid == 0) piv_of[k] = (short)piv;
+            if (tid == 0) {
+                piv_of[k] = (short)piv;
+                lam[k] = d;
+            }
             __syncthreads();
-            for (int e = tid; e < nq * ROWS; e += NT) {   // a warp works on one column
-                const int q = e / ROWS, i = e % ROWS;
-                const int j = crank + C * q;
-                const T lj = lk[j];
-                if (i >= M || lj == T(0) || j == piv) continue;   // l is zero on the rows of earlier pivots
-                const T v = fma(-lk[i], lj, A[q * LD + i]);
-                A[q * LD + i] = v;
-                if (i == j) dg[q] = v;
+#pragma unroll
+            for (int q = 0; q < QT; ++q) {
+                const int cq = cg + CT * q, j = crank + C * cq;
+                if (cq >= NQ || j >= M) break;
+                const T lj = lk[j];   // zero for the columns of earlier pivots
+                if (__double2hiint(lj) == 0 || j == piv) continue;
+#pragma unroll
+                for (int a = 0; a < RT; ++a) {
+                    const int i = row + a * NT;
+                    Ar[a][q] = fma(col[a], lj, Ar[a][q]);
+                    if (i < ROWS) A[cq * LD + i] = Ar[a][q];
+                    if (i == j) dg[cq] = Ar[a][q];
+                }
             }
             if (own == crank && tid == 0) dg[q0] = T(-1);
             __syncthreads();
@@ -395,6 +428,7 @@ __global__ void __launch_bounds__(SH::NT, 1)
         // FP32 arithmetic is cheaper than the cluster's barrier: every CTA factorises the whole Gram, held in registers
         // (entry (i, j) with j = warp + NW a, i = lane + 32 b), and keeps its own columns
         constexpr int NW = NT / 32, NA = ROWS / NW, NB = ROWS / 32;
+        static_assert(NW == 16, "two columns of a warp to a row block");
         float Ar[NA][NB];
 #pragma unroll
         for (int a = 0; a < NA; ++a)
@@ -403,10 +437,11 @@ __global__ void __launch_bounds__(SH::NT, 1)
                 const int i = lane + 32 * b, j = warp + NW * a;
                 Ar[a][b] = (i < M && j < M) ? G[i + (long long)j * M] * sc : 0.f;
             }
-        for (int i = tid; i < ROWS; i += NT) dgf[i] = i < M ? G[i + (long long)i * M] * sc : -1.f;
+        for (int i = tid; i < ROWS; i += NT) dgf[i] = i < M ? G[i + (long long)i * M] * sc : 0.f;
         __syncthreads();
         const float thr = 1e-9f * tr;
         const float stop_rem = fmaxf(thr, 0.01f * (float)bus);
+        unsigned dead_row = 0, dead_col = 0;   // pivoted ones among this lane's rows (bit b) and this warp's columns (bit a)
         for (int k = 0; k < M; ++k) {
             // the largest remaining diagonal entry (ties: the lowest index) and the remaining trace, in every warp
             float v = -2.f, sm = 0.f;
@@ -425,20 +460,25 @@ __global__ void __launch_bounds__(SH::NT, 1)
             if (best < 0 || !(sm > stop_rem)) break;   // the same decision in every thread and CTA
             float* lk = lbuf[k & 1];
             if (warp == piv % NW) {
-                const float r = __fsqrt_rn(__int_as_float(best));
+                // l = A[:, piv] / sqrt(d), zero on the rows of earlier pivots.  (An IEEE square root and divisions here kept
+                // the other warps waiting for 1000 of 2500 cycles a step.)
+                const float d = __int_as_float(best), y0 = rsqrtf(d);
+                const float inv = fmaf(y0 * fmaf(-d * y0, y0, 1.f), 0.5f, y0);
                 const int ap = piv / NW;
-                T* out = k % C == crank ? S + (long long)k * n : nullptr;
+                float* out = k % C == crank ? S + (long long)k * n : nullptr;
 #pragma unroll
                 for (int b = 0; b < NB; ++b) {
                     float a = 0.f;
 #pragma unroll
                     for (int q = 0; q < NA; ++q) a = (q == ap) ? Ar[q][b] : a;
                     const int i = lane + 32 * b;
-                    a = (i == piv) ? r : __fdiv_rn(a, r);
+                    a = dead_row >> b & 1 ? 0.f : a * inv;
                     lk[i] = a;
                     if (out && i < M) out[i] = a;
                 }
+                dead_col |= 1u << ap;
             }
+            if (lane == (piv & 31)) dead_row |= 1u << (piv >> 5);
             __syncthreads();
             float li[NB];
 #pragma unroll
@@ -448,12 +488,9 @@ __global__ void __launch_bounds__(SH::NT, 1)
                 const int j = warp + NW * a;
                 const float lj = lk[j];
 #pragma unroll
-                for (int b = 0; b < NB; ++b) {
-                    const int i = lane + 32 * b;
-                    const float w = (i == piv || j == piv) ? 0.f : fmaf(-li[b], lj, Ar[a][b]);
-                    Ar[a][b] = w;
-                    if (i == j && i < M) dgf[i] = (i == piv || dgf[i] < 0.f) ? -1.f : w;
-                }
+                for (int b = 0; b < NB; ++b) Ar[a][b] = fmaf(-li[b], lj, Ar[a][b]);
+                // column j's diagonal is in register b = a / 2 of one lane (0 once pivoted)
+                if (lane == warp + NW * (a & 1)) dgf[j] = dead_col >> a & 1 ? 0.f : Ar[a][a >> 1];
             }
             __syncthreads();
             rc = k + 1;
@@ -466,16 +503,23 @@ __global__ void __launch_bounds__(SH::NT, 1)
     const int Ce = max(1, min(C, (rc + 2 * SH::BT - 1) / (2 * SH::BT)));
     const int b = crank < Ce ? max(1, ((rc + Ce - 1) / Ce + 1) / 2) : 0;
     const int grp = tid / LPP, gl = tid % LPP;
+    int set = sizeof(T) == 8 ? 1 : 0, nsweeps = 0;
     for (int e = tid; e < 2 * b * ROWS; e += NT) {
         const int i = e % ROWS, slot = e / ROWS, k = slot * Ce + crank;
-        cols[((slot & 1) * BMAX + (slot >> 1)) * LD + i] = k < rc && i < M ? S[i + (long long)k * n] : T(0);
+        T v = T(0);
+        if constexpr (sizeof(T) == 8) {   // from where the Cholesky left it, scaled by the pivot (kept by every CTA)
+            if (k < rc) v = cluster.map_shared_rank(cols, k % C)[(k / C) * LD + i] * hj_rsqrt(lam[k]);
+        } else {
+            if (k < rc && i < M) v = S[i + (long long)k * n];
+        }
+        cols[((2 * set + (slot & 1)) * BMAX + (slot >> 1)) * LD + i] = v;
     }
-    __syncthreads();
+    if constexpr (sizeof(T) == 8) cluster.sync();   // read by everybody before the blocks move
+    else __syncthreads();
     const T skip = sizeof(T) == 8 && !p.strict ? (T)(1e-3 * bus * (double)__fdividef(1.f, (float)M)) : T(0);
     // (a direction of discarded energy below budget / (M + 1) in all is discarded with any basis of it)
     const T floor_g = sizeof(T) == 8 ? T(0) : T(1e-12f) * tr;   // FP32 products below this are noise of the factor
     auto column = [&](int set, int blk, int pos) -> T* { return cols + ((set * 2 + blk) * BMAX + pos) * LD; };
-    int set = 0, nsweeps = 0;
     T x[RPL], y[RPL];
     for (int sweep = 0; sweep < max_sweeps && rc > 1; ++sweep) {
         ++nsweeps;
@@ -615,20 +659,31 @@ __global__ void __launch_bounds__(SH::NT, 1)
             for (int r = 0; r < C; ++r) cluster.map_shared_rank(lam, r)[k] = (double)s;
     }
     cluster.sync();
-    for (int i = tid; i < M; i += NT) {   // squared norms are not negative: their bits order as integers
+    // ranks by counting: squared norms are not negative, so their bits order as integers (32 of them in FP32)
+    using K = typename std::conditional<sizeof(T) == 8, long long, int>::type;
+    K* keys = reinterpret_cast<K*>(lbuf);
+    for (int i = tid; i < ROWS; i += NT) {
+        K key = -1;
         if (i < rc) {
             const double v = lam[i];
-            const long long li = v == v ? __double_as_longlong(v) : -1;
-            int rk = 0;
-            for (int j = 0; j < rc; ++j) {
-                const double w = lam[j];
-                const long long lj = w == w ? __double_as_longlong(w) : -1;
-                rk += (lj > li || (lj == li && j < i)) ? 1 : 0;
-            }
+            if constexpr (sizeof(T) == 8) key = v == v ? __double_as_longlong(v) : -1;
+            else key = v == v ? __float_as_int((float)v) : -1;
+        }
+        keys[i] = key;
+        if (i >= rc && i < M) lsort[i] = 0.0;
+    }
+    __syncthreads();
+    // (four lanes per player)
+    for (int e = tid; e < 4 * ROWS; e += NT) {
+        const int i = e >> 2;
+        int rk = 0;
+        const K own = keys[i];
+        for (int j = e & 3; j < rc; j += 4) rk += (keys[j] > own || (keys[j] == own && j < i)) ? 1 : 0;
+        rk += __shfl_xor_sync(FULL, rk, 1);
+        rk += __shfl_xor_sync(FULL, rk, 2);
+        if (i < rc && (e & 3) == 0) {
             ord[i] = (short)rk;
-            lsort[rk] = v * unscale;
-        } else {
-            lsort[i] = 0.0;
+            lsort[rk] = lam[i] * unscale;
         }
     }
     __syncthreads();

@@ -10,7 +10,7 @@
 // 111 / 60 / 33 us on four CTAs of 16 warps (one CTA of 32 warps 158 / 81 / 36, eight of 16 98 / 57 / 32); FP64 453 / 222 / 112 us
 // on eight CTAs of 8 warps (eight of 4 532 / 259 / 111, sixteen of 4 435 / 223 / 113).  The kernel this replaces, one CTA with
 // its working copy in global memory, took 400 us in FP32 at 106 columns and 190 us in FP64 for 17 columns at n = 32 (now 41).
-//  Reflectors are kept unscaled, H = I - f v v^T with v = a -+ |a| e_1 and f = 1 / (|a| (|a| + |a_1|)).
+// Reflectors are kept unscaled, H = I - f v v^T with v = a -+ |a| e_1 and f = 1 / (|a| (|a| + |a_1|)).
 #include <math.h>
 
 #include <mutex>
