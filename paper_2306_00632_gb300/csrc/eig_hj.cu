@@ -19,9 +19,9 @@
 // instructions for one pair).  Hence one pair per quarter, on as many CTAs as the columns fill so; shears with three
 // FMAs an element; everything that only steers the iteration in FP32; and no rotation of pairs far below the budget.
 // Measured, FP64, a Gram of order 120 and full rank: 1.5 ms (16 CTAs), where the two-sided cyclic Jacobi on 8 CTAs that
-// this replaces took 18 ms at order 97; order 32: 0.22 ms against 0.8 ms.  FP32, where a step is 0.4 us of latencies: order
-// 120 and full rank 0.29 ms (four CTAs), rank 51 0.13 ms, rank 16 0.04 ms, where a ring of columns in one CTA's registers
-// with a barrier a step took 0.92, 0.19 and 0.06 ms.
+// this replaces took 18 ms at order 97; order 32: 0.22 ms against 0.8 ms.  FP32, where a step is latency and instructions
+// (0.3 us with 16-byte accesses and paired FMAs, 0.45 us without): order 128 and rank 45 0.14 ms, where a ring of columns in
+// one CTA's registers with a barrier a step took 0.43 ms.
 #include <math.h>
 
 #include <mutex>
@@ -87,6 +87,32 @@ __device__ __forceinline__ double hj_rsqrt(double d) {
     return fma(y * e, fma(e, 0.375, 0.5), y);
 }
 
+// This lane's rows of a column at a: rows gl + LPP q, the first rpl of them; in FP32 with a warp per pair the four rows
+// 4 gl + q in one 16-byte access (all of them: rows past the order are zero, and an FP32 FMA is cheaper than a test)
+template <typename T, int LPP, int RPL>
+constexpr bool hj_vec = sizeof(T) == 4 && LPP == 32 && RPL == 4;
+template <typename T, int LPP, int RPL>
+__device__ __forceinline__ void hj_load(T (&x)[RPL], const T* a, int gl, int rpl) {
+    if constexpr (hj_vec<T, LPP, RPL>) {
+        const float4 v = *reinterpret_cast<const float4*>(a + 4 * gl);
+        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+    } else {
+#pragma unroll
+        for (int q = 0; q < RPL; ++q)
+            if (q < rpl) x[q] = a[gl + LPP * q];
+    }
+}
+template <typename T, int LPP, int RPL>
+__device__ __forceinline__ void hj_save(const T (&x)[RPL], T* a, int gl, int rpl) {
+    if constexpr (hj_vec<T, LPP, RPL>) {
+        *reinterpret_cast<float4*>(a + 4 * gl) = make_float4(x[0], x[1], x[2], x[3]);
+    } else {
+#pragma unroll
+        for (int q = 0; q < RPL; ++q)
+            if (q < rpl) a[gl + LPP * q] = x[q];
+    }
+}
+
 // One pair: x and y are this lane's rows of the two columns (zero for an idle group), ax and ay their squared norms.
 // Whole warps call it.  A pair with |x . y| above tau |x| |y| is rotated: u = tan(theta / 2), s = sin(theta), applied
 // as the shears x -= u y, y += s x, x -= u y (three FMAs an element).  The angle needs no more than FP32: an error of
@@ -95,9 +121,15 @@ __device__ __forceinline__ double hj_rsqrt(double d) {
 template <typename T, int LPP, int RPL>
 __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, int rpl, T skip, T floor_g, int& big) {
     T g = T(0);
+    if constexpr (hj_vec<T, LPP, RPL>) {
+        const float2 g2 = __ffma2_rn(make_float2(x[2], x[3]), make_float2(y[2], y[3]),
+                                     __fmul2_rn(make_float2(x[0], x[1]), make_float2(y[0], y[1])));
+        g = g2.x + g2.y;
+    } else {
 #pragma unroll
-    for (int q = 0; q < RPL; ++q)
-        if (q < rpl) g = fma(x[q], y[q], g);
+        for (int q = 0; q < RPL; ++q)
+            if (q < rpl) g = fma(x[q], y[q], g);
+    }
 #pragma unroll
     for (int o = LPP / 2; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
     float fa, fb, fg, fd;   // |x|^2, |y|^2, x . y, |y|^2 - |x|^2
@@ -118,11 +150,11 @@ __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, 
         fd = ay - ax;
         on = fabsf(g) > floor_g;
     }
-    // t = tan(theta) = sign(d g) 2 |g| / (|d| + sqrt(d^2 + 4 g^2)); u = t / (1 + sqrt(1 + t^2)), its series in t^2 fitted
-    // on [0, 1] to 2e-6.  Formed beside the test, not after it.
-    const float ab = fa * fb, ag = fabsf(fg);
-    const float h = fmaf(fd, fd, 4.f * fg * fg);
-    const float t = copysignf(1.f, fd) * __fdividef(2.f * fg, fmaf(h, rsqrtf(h), fabsf(fd)));
+    // t = tan(theta) = 2 g / (d + sign(d) sqrt(d^2 + 4 g^2)); u = t / (1 + sqrt(1 + t^2)), its series in t^2 fitted on
+    // [0, 1] to 2e-6.  Formed beside the test, not after it.
+    const float ab = fa * fb, ag = fabsf(fg), f2g = 2.f * fg;
+    const float h = fmaf(fd, fd, f2g * f2g);
+    const float t = __fdividef(f2g, fd + copysignf(h * rsqrtf(h), fd));
     const float w = t * t;
     const float u = t * fmaf(w, fmaf(w, fmaf(w, fmaf(w, fmaf(w, -0.00342296f, 0.0151217f), -0.03403639f), 0.06147052f),
                              -0.12491905f), 0.49999894f);
@@ -135,7 +167,7 @@ __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, 
         above = ag * ag > hj_tau<T>() * hj_tau<T>() * ab;
         large = ag * ag > hj_last<T>() * hj_last<T>() * ab;
     }
-    if (on && above && fabsf(u) > 1e-30f) {
+    if (on && above && (sizeof(T) == 4 || fabsf(u) > 1e-30f)) {
         if (large) big = 1;
         T ud, s;
         if constexpr (sizeof(T) == 8) {
@@ -154,13 +186,26 @@ __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, 
             const float q = fmaf(u, u, 1.f), r0 = __fdividef(1.f, q);
             s = 2.f * u * fmaf(r0, fmaf(-q, r0, 1.f), r0);
         }
+        if constexpr (hj_vec<T, LPP, RPL>) {
+            const float2 mu = make_float2(-u, -u), s2 = make_float2(s, s);
 #pragma unroll
-        for (int q = 0; q < RPL; ++q)
-            if (q < rpl) {
-                const T x1 = fma(-ud, y[q], x[q]);
-                y[q] = fma(s, x1, y[q]);
-                x[q] = fma(-ud, y[q], x1);
+            for (int q = 0; q < 4; q += 2) {
+                float2 yq = make_float2(y[q], y[q + 1]);
+                const float2 x1 = __ffma2_rn(mu, yq, make_float2(x[q], x[q + 1]));
+                yq = __ffma2_rn(s2, x1, yq);
+                const float2 xq = __ffma2_rn(mu, yq, x1);
+                x[q] = xq.x; x[q + 1] = xq.y;
+                y[q] = yq.x; y[q + 1] = yq.y;
             }
+        } else {
+#pragma unroll
+            for (int q = 0; q < RPL; ++q)
+                if (q < rpl) {
+                    const T x1 = fma(-ud, y[q], x[q]);
+                    y[q] = fma(s, x1, y[q]);
+                    x[q] = fma(-ud, y[q], x1);
+                }
+        }
         const float tg = t * fg;   // the norms are exact again at the next sweep
         if constexpr (sizeof(T) == 8) {
             if (fabsf(tg) > 1e-30f) {
@@ -228,6 +273,7 @@ __global__ void __launch_bounds__(SH::NT, 1)
     constexpr int NQ = 2 * BMAX;                    // columns of G per CTA (Cholesky)
     constexpr unsigned FULL = 0xffffffffu;
     static_assert(NQ <= 32, "one lane per column in the search for the pivot");
+    static_assert(LPP == 32, "a warp per pair: no warp holds a pair beside an idle one");
     cgx::cluster_group cluster = cgx::this_cluster();
     const int crank = (int)cluster.block_rank();
     RoundPlan& p = *plan;
@@ -527,10 +573,10 @@ __global__ void __launch_bounds__(SH::NT, 1)
         for (int blk = 0; blk < 2; ++blk) {   // exact squared norms
             T s = T(0);
             if (grp < b) {
-                const T* a = column(set, blk, grp);
+                hj_load<T, LPP, RPL>(x, column(set, blk, grp), gl, rpl);
 #pragma unroll
                 for (int q = 0; q < RPL; ++q)
-                    if (q < rpl) { const T v = a[gl + LPP * q]; s = fma(v, v, s); }
+                    if (q < rpl || hj_vec<T, LPP, RPL>) s = fma(x[q], x[q], s);
             }
 #pragma unroll
             for (int o = LPP / 2; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
@@ -555,47 +601,41 @@ __global__ void __launch_bounds__(SH::NT, 1)
             }
             const bool on = i >= 0;
             if (__any_sync(FULL, on)) {
-                T* xp = column(set, on ? blk : 0, on ? i : 0) + gl;
-                T* yp = column(set, on ? blk : 0, on ? j : 0) + gl;
+                T* xp = column(set, on ? blk : 0, on ? i : 0);
+                T* yp = column(set, on ? blk : 0, on ? j : 0);
                 T ax = on ? nrm[set][blk][i] : T(0), ay = on ? nrm[set][blk][j] : T(0);
-#pragma unroll
-                for (int q = 0; q < RPL; ++q)
-                    if (q < rpl) { x[q] = on ? xp[LPP * q] : T(0); y[q] = on ? yp[LPP * q] : T(0); }
+                hj_load<T, LPP, RPL>(x, xp, gl, rpl);
+                hj_load<T, LPP, RPL>(y, yp, gl, rpl);
                 hj_pair<T, LPP, RPL>(x, y, ax, ay, rpl, skip, floor_g, big);
                 if (on) {
-#pragma unroll
-                    for (int q = 0; q < RPL; ++q)
-                        if (q < rpl) { xp[LPP * q] = x[q]; yp[LPP * q] = y[q]; }
+                    hj_save<T, LPP, RPL>(x, xp, gl, rpl);
+                    hj_save<T, LPP, RPL>(y, yp, gl, rpl);
                     if (gl == 0) { nrm[set][blk][i] = ax; nrm[set][blk][j] = ay; }
                 }
             }
             __syncthreads();
         }
         for (int round = 0; round < 2 * Ce - 1; ++round) {
-            const bool act = grp < b;
-            const bool wact = warp * (32 / LPP) < b;   // this warp has a pair (b is 0 where the CTA has none)
+            const bool act = grp < b;   // (b is 0 where the CTA has no columns; a warp with no pair at all skips the steps)
+            const bool wact = LPP == 32 ? act : warp * (32 / LPP) < b;
             T ax = T(0);
             if (wact) {
-                const T* xp = column(set, 0, act ? grp : 0) + gl;
+                hj_load<T, LPP, RPL>(x, column(set, 0, act ? grp : 0), gl, rpl);
                 ax = act ? nrm[set][0][grp] : T(0);
-#pragma unroll
-                for (int q = 0; q < RPL; ++q)
-                    if (q < rpl) x[q] = act ? xp[LPP * q] : T(0);
             }
+            int j = grp;
+            T* yp = column(set, 1, act ? grp : 0);
             for (int k = 0; k < b; ++k) {
                 if (wact) {
-                    int j = grp + k; if (j >= b) j -= b;
-                    T* yp = column(set, 1, act ? j : 0) + gl;
                     T ay = act ? nrm[set][1][j] : T(0);
-#pragma unroll
-                    for (int q = 0; q < RPL; ++q)
-                        if (q < rpl) y[q] = act ? yp[LPP * q] : T(0);
+                    hj_load<T, LPP, RPL>(y, yp, gl, rpl);
                     hj_pair<T, LPP, RPL>(x, y, ax, ay, rpl, skip, floor_g, big);
                     if (act) {
-#pragma unroll
-                        for (int q = 0; q < RPL; ++q)
-                            if (q < rpl) yp[LPP * q] = y[q];
+                        hj_save<T, LPP, RPL>(y, yp, gl, rpl);
                         if (gl == 0) nrm[set][1][j] = ay;
+                        ++j;
+                        yp += LD;
+                        if (j == b) { j = 0; yp -= b * LD; }
                     }
                 }
                 __syncthreads();
@@ -606,10 +646,7 @@ __global__ void __launch_bounds__(SH::NT, 1)
             }
             if (Ce == 1) {
                 if (act) {
-                    T* xp = column(set, 0, grp) + gl;
-#pragma unroll
-                    for (int q = 0; q < RPL; ++q)
-                        if (q < rpl) xp[LPP * q] = x[q];
+                    hj_save<T, LPP, RPL>(x, column(set, 0, grp), gl, rpl);
                     if (gl == 0) nrm[set][0][grp] = ax;
                 }
                 cluster.sync();
@@ -621,19 +658,13 @@ __global__ void __launch_bounds__(SH::NT, 1)
             const int tb = crank == 0 ? 0 : (crank == Ce - 1 ? 1 : 0);
             const int bc = crank == 0 ? 1 : crank - 1, bb = crank == 0 ? 0 : 1;
             if (act) {
-                T* dst = cluster.map_shared_rank(cols, tc) + ((ns * 2 + tb) * BMAX + grp) * LD + gl;
-#pragma unroll
-                for (int q = 0; q < RPL; ++q)
-                    if (q < rpl) dst[LPP * q] = x[q];
+                hj_save<T, LPP, RPL>(x, cluster.map_shared_rank(cols, tc) + ((ns * 2 + tb) * BMAX + grp) * LD, gl, rpl);
                 if (gl == 0) {
                     cluster.map_shared_rank(&nrm[0][0][0], tc)[(ns * 2 + tb) * BMAX + grp] = ax;
                     cluster.map_shared_rank(&nrm[0][0][0], bc)[(ns * 2 + bb) * BMAX + grp] = nrm[set][1][grp];
                 }
-                T* dsb = cluster.map_shared_rank(cols, bc) + ((ns * 2 + bb) * BMAX + grp) * LD + gl;
-                const T* yb = column(set, 1, grp) + gl;
-#pragma unroll
-                for (int q = 0; q < RPL; ++q)
-                    if (q < rpl) dsb[LPP * q] = yb[LPP * q];
+                hj_load<T, LPP, RPL>(y, column(set, 1, grp), gl, rpl);
+                hj_save<T, LPP, RPL>(y, cluster.map_shared_rank(cols, bc) + ((ns * 2 + bb) * BMAX + grp) * LD, gl, rpl);
             }
             cluster.sync();
             set = ns;
@@ -647,10 +678,10 @@ __global__ void __launch_bounds__(SH::NT, 1)
     for (int blk = 0; blk < 2; ++blk) {
         T s = T(0);
         if (grp < b) {
-            const T* a = column(set, blk, grp);
+            hj_load<T, LPP, RPL>(x, column(set, blk, grp), gl, rpl);
 #pragma unroll
             for (int q = 0; q < RPL; ++q)
-                if (q < rpl) { const T v = a[gl + LPP * q]; s = fma(v, v, s); }
+                if (q < rpl || hj_vec<T, LPP, RPL>) s = fma(x[q], x[q], s);
         }
 #pragma unroll
         for (int o = LPP / 2; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
