@@ -43,42 +43,48 @@ int set_zero(tucker_t* t, cudaStream_t st) { return set_plain(t, 0, 0, 0, st); }
 // --------------------------------------------------------------------------------------------------
 constexpr int APPLY_CB = 8;
 
-// output descriptor of the apply: blocks (f) + (j, b) for every term j and input block b
+// Output descriptor of the apply: blocks (f) + (j, b) for every term j and input block b.  Called by one whole block: the
+// threads write one block each (one thread that walked over them took most of the launch at 19 terms).  For an append yd
+// is fdsc: everything is read before anything is written.
 __device__ void apply_desc(const TuckerDesc* __restrict__ xd, const double* __restrict__ w, int R, double sign,
                            const TuckerDesc* fdsc, TuckerDesc* yd, int cap, int* err, double* prof, int n, int p,
                            int elt) {
-    if (prof) {   // algorithmic work of the banded products: bands read once, X read, Y written
+    const int tid = threadIdx.x, nt = blockDim.x;
+    if (prof && tid == 0) {   // algorithmic work of the banded products: bands read once, X read, Y written
         double cols = (double)xd->rank[0] + xd->rank[1] + xd->rank[2];
         prof[2 * PK_APPLY] += 2.0 * (2 * p + 1) * (double)n * R * cols;
         prof[2 * PK_APPLY + 1] += (double)elt * ((double)R * 3 * (2 * p + 1) * n + (double)n * cols * (1.0 + R));
     }
-    int nb = 0;
+    // leading blocks: the rhs (residual) or y itself (append; fdsc == yd, nothing to copy)
+    const int nb = fdsc ? fdsc->nblk : 0, nx = xd->nblk;
     int base[3] = {0, 0, 0};
-    if (fdsc) {   // leading blocks: the rhs (residual) or y itself (append; fdsc == yd, nothing to copy)
+    if (fdsc)
         for (int t = 0; t < 3; ++t) base[t] = fdsc->rank[t];
-        if (fdsc == yd)
-            nb = fdsc->nblk;
-        else
-            for (int b = 0; b < fdsc->nblk; ++b) yd->blk[nb++] = fdsc->blk[b];
-    }
     const int kx[3] = {xd->rank[0], xd->rank[1], xd->rank[2]};
-    bool ok = (nb + R * xd->nblk <= TPCG_MAX_BLOCKS);
+    bool ok = (nb + R * nx <= TPCG_MAX_BLOCKS);
     for (int t = 0; t < 3; ++t) ok = ok && (base[t] + (long long)R * kx[t] <= cap);
+    __syncthreads();
     if (!ok) {
-        if (err) *err = 1;
-        yd->nblk = 0;
-        yd->rank[0] = yd->rank[1] = yd->rank[2] = 0;
+        if (tid == 0) {
+            if (err) *err = 1;
+            yd->nblk = 0;
+            yd->rank[0] = yd->rank[1] = yd->rank[2] = 0;
+        }
         return;
     }
-    for (int j = 0; j < R; ++j)
-        for (int b = 0; b < xd->nblk; ++b) {
-            BlockDesc B = xd->blk[b];
-            for (int t = 0; t < 3; ++t) B.off[t] += base[t] + j * kx[t];
-            B.scale *= sign * w[j];
-            yd->blk[nb++] = B;
-        }
-    yd->nblk = nb;
-    for (int t = 0; t < 3; ++t) yd->rank[t] = base[t] + R * kx[t];
+    if (fdsc != yd)
+        for (int b = tid; b < nb; b += nt) yd->blk[b] = fdsc->blk[b];
+    for (int e = tid; e < R * nx; e += nt) {
+        const int j = e / nx, b = e % nx;
+        BlockDesc B = xd->blk[b];
+        for (int t = 0; t < 3; ++t) B.off[t] += base[t] + j * kx[t];
+        B.scale *= sign * w[j];
+        yd->blk[nb + e] = B;
+    }
+    if (tid == 0) {
+        yd->nblk = nb + R * nx;
+        for (int t = 0; t < 3; ++t) yd->rank[t] = base[t] + R * kx[t];
+    }
 }
 
 // yd: when non-null, block (0, 0, 0) also writes the output descriptor (only when yd is not read by this kernel,
@@ -92,7 +98,7 @@ __global__ void __launch_bounds__(128) apply_kernel(const T* __restrict__ bands,
                                                     const T* F2, TuckerDesc* yd, const double* __restrict__ w,
                                                     double sign, int* err, double* prof) {
     constexpr int BW = 2 * P + 1;
-    if (yd && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0)
+    if (yd && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)
         apply_desc(xd, w, R, sign, fd, yd, cap, err, prof, n, P, (int)sizeof(T));
     const int t = blockIdx.z, j = blockIdx.y / nchunk, chunk = blockIdx.y % nchunk;
     const int i0 = blockIdx.x * blockDim.x;
@@ -171,7 +177,6 @@ static int launch_apply(int p, dim3 grid, cudaStream_t st, const T* bands, int n
 __global__ void apply_desc_kernel(const TuckerDesc* __restrict__ xd, const double* __restrict__ w, int R,
                                   double sign, const TuckerDesc* fdsc, TuckerDesc* yd, int cap,
                                   int* err, double* prof, int n, int p, int elt) {
-    if (threadIdx.x != 0) return;
     apply_desc(xd, w, R, sign, fdsc, yd, cap, err, prof, n, p, elt);
 }
 
@@ -217,7 +222,7 @@ int apply_append_impl(tpcg_problem pb, const tucker_t* x, tucker_t* y, double si
                              static_cast<T*>(y->U[1]), static_cast<T*>(y->U[2]), y->cap,
                              static_cast<const TuckerDesc*>(y->desc), nullptr, nullptr, nullptr, nullptr, nullptr,
                              0.0, nullptr, nullptr));
-    apply_desc_kernel<<<1, 32, 0, st>>>(static_cast<const TuckerDesc*>(x->desc), pb->d_w, pb->R, sign,
+    apply_desc_kernel<<<1, TPCG_MAX_BLOCKS, 0, st>>>(static_cast<const TuckerDesc*>(x->desc), pb->d_w, pb->R, sign,
                                         static_cast<const TuckerDesc*>(y->desc), static_cast<TuckerDesc*>(y->desc),
                                         y->cap, err, prof_dev(), n, pb->p, (int)sizeof(T));
     TPCG_CHECK_LAUNCH();
@@ -662,31 +667,35 @@ __global__ void fd_scatter_kernel(const TuckerDesc* __restrict__ sd, const T* A0
 __global__ void fd_desc_kernel(const TuckerDesc* __restrict__ sd, const double* __restrict__ omega, double lmin,
                                int RP, TuckerDesc* vd, int vcap, int* err, double* prof, int n, int n1, int n2, int p,
                                int elt) {
-    if (threadIdx.x != 0) return;
-    if (prof) {   // algorithmic work of Alg. 4 per input column: W^T gather, sine transforms, R_P scalings, W scatter
+    const int tid = threadIdx.x;   // a thread per block
+    if (prof && tid == 0) {   // algorithmic work of Alg. 4 per input column: W^T gather, sine transforms, R_P scalings, W scatter
         const double cols = (double)sd->rank[0] + sd->rank[1] + sd->rank[2];
         const double lg = n1 > 1 ? log2((double)n1) : 1.0;
         prof[2 * PK_FD] += (1.0 + RP) * cols * (5.0 * n1 * lg + 4.0 * (p + 1) * n + 2.0 * (double)n * n2);
         prof[2 * PK_FD + 1] += (double)elt * (double)n * cols * (2.0 + 2.0 * RP);
     }
-    bool ok = RP * sd->nblk <= TPCG_MAX_BLOCKS;
+    const int ns = sd->nblk;
+    bool ok = RP * ns <= TPCG_MAX_BLOCKS;
     for (int t = 0; t < 3; ++t) ok = ok && (RP * sd->rank[t] <= vcap);
     if (!ok) {
-        if (err) *err = 1;
-        vd->nblk = 0;
-        vd->rank[0] = vd->rank[1] = vd->rank[2] = 0;
+        if (tid == 0) {
+            if (err) *err = 1;
+            vd->nblk = 0;
+            vd->rank[0] = vd->rank[1] = vd->rank[2] = 0;
+        }
         return;
     }
-    int nb = 0;
-    for (int j = 0; j < RP; ++j)
-        for (int b = 0; b < sd->nblk; ++b) {
-            BlockDesc B = sd->blk[b];
-            for (int t = 0; t < 3; ++t) B.off[t] += j * sd->rank[t];
-            B.scale *= omega[j] / lmin;
-            vd->blk[nb++] = B;
-        }
-    vd->nblk = nb;
-    for (int t = 0; t < 3; ++t) vd->rank[t] = RP * sd->rank[t];
+    for (int e = tid; e < RP * ns; e += blockDim.x) {
+        const int j = e / ns, b = e % ns;
+        BlockDesc B = sd->blk[b];
+        for (int t = 0; t < 3; ++t) B.off[t] += j * sd->rank[t];
+        B.scale *= omega[j] / lmin;
+        vd->blk[e] = B;
+    }
+    if (tid == 0) {
+        vd->nblk = RP * ns;
+        for (int t = 0; t < 3; ++t) vd->rank[t] = RP * sd->rank[t];
+    }
 }
 
 template <typename T>
@@ -749,7 +758,7 @@ int fd_impl(tpcg_problem pb, tpcg_ctx c, const tucker_t* s, tucker_t* v, cudaStr
                                              static_cast<T*>(v->U[1]), static_cast<T*>(v->U[2]), v->cap);
     TPCG_CHECK_LAUNCH();
     if (n2 > 0) TPCG_TRY((launch_gemm<T, false, false>(ga + 9, counts, 3, 1, n, RP * rc, st)));
-    fd_desc_kernel<<<1, 32, 0, st>>>(sd, pb->d_omega, lmin, RP, static_cast<TuckerDesc*>(v->desc), v->cap,
+    fd_desc_kernel<<<1, TPCG_MAX_BLOCKS, 0, st>>>(sd, pb->d_omega, lmin, RP, static_cast<TuckerDesc*>(v->desc), v->cap,
                                      err, prof_dev(), n, n1, n2, pb->p, (int)sizeof(T));
     TPCG_CHECK_LAUNCH();
     prof_end(PK_FD, st);

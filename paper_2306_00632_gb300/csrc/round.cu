@@ -28,12 +28,18 @@ namespace tpcg {
 // Planner: descriptor -> plan and the GEMM arguments of step 2.
 // gargs layout: [0, MAXB) middle-mode products, [MAXB, 2 MAXB) mode-1 products, [2 MAXB] fused mode 3.
 // --------------------------------------------------------------------------------------------------
+constexpr int PLAN_THREADS = 128;
+static_assert(PLAN_THREADS >= TPCG_MAX_BLOCKS && PLAN_THREADS >= MAX_SPLIT, "one thread per block or partial Gram");
+
 template <typename T>
-__global__ void plan_round_kernel(const TuckerDesc* __restrict__ d, RoundPlan* plan, GemmArgs* ga, int n,
+__global__ void __launch_bounds__(PLAN_THREADS) plan_round_kernel(const TuckerDesc* __restrict__ d, RoundPlan* plan, GemmArgs* ga, int n,
                                   int cap, double eps_host, const double* eps_dev, void* Rq0, void* Rq1,
                                   void* Rq2, const void* U0, const void* U1, const void* U2, T* T1, T* Wm,
                                   int* counts, long long t1cap, double* prof, int strict_mode, void* Zout) {
-    if (threadIdx.x != 0) return;
+    // thread b plans block b (PLAN_THREADS >= TPCG_MAX_BLOCKS): one thread walking over the blocks waited for a read of
+    // global memory per block, 8 us for 19 of them
+    __shared__ long long wsum[PLAN_THREADS / 32];
+    const int b = threadIdx.x, lane = b & 31, warp = b >> 5;
     RoundPlan p;
     p.n = n;
     p.nblk = d->nblk;
@@ -61,56 +67,70 @@ __global__ void plan_round_kernel(const TuckerDesc* __restrict__ d, RoundPlan* p
     p.kz3 = p.k[2];
     p.nsplit = 0;
     const int kp1 = p.kp[0], kp2 = p.kp[1];
+    BlockDesc B{};
+    if (b < p.nblk) B = d->blk[b];
+    const int r1 = B.r[0], r2 = B.r[1], r3 = B.r[2];
+    const bool empty = r1 == 0 || r2 == 0 || r3 == 0;
+    long long off = (long long)r1 * kp2 * r3;   // the blocks' places in T1, one after the other
+    const long long own = off;
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long v = __shfl_up_sync(0xffffffffu, off, o);
+        if (lane >= o) off += v;
+    }
+    if (lane == 31) wsum[warp] = off;
+    __syncthreads();
     long long t1off = 0;
-    for (int b = 0; b < p.nblk; ++b) {
-        const BlockDesc& B = d->blk[b];
-        const int r1 = B.r[0], r2 = B.r[1], r3 = B.r[2];
+    for (int w = 0; w < PLAN_THREADS / 32; ++w) {
+        if (w < warp) off += wsum[w];
+        t1off += wsum[w];
+    }
+    off -= own;
+    if (b < p.nblk) {
         // middle mode on the core: U_b[:, :, j3] (r1 x kp2) = G_b[:, :, j3] (r1 x r2) R_2b^T
         GemmArgs a{};
         a.M = r1; a.N = kp2; a.K = r2; a.nbatch = r3; a.acc = 0;
         a.A = B.core; a.lda = r1; a.sA = (long long)r1 * r2;
         a.B = static_cast<const T*>(p.Rp[1]) + (long long)B.off[1] * p.ldR[1]; a.ldb = p.ldR[1]; a.sB = 0;
-        a.C = T1 + t1off; a.ldc = r1; a.sC = (long long)r1 * kp2;
+        a.C = T1 + off; a.ldc = r1; a.sC = (long long)r1 * kp2;
         a.alpha = 1.0; a.beta = 0.0;
-        if (r1 == 0 || r2 == 0 || r3 == 0) { a.M = 0; a.nbatch = 0; }
+        if (empty) { a.M = 0; a.nbatch = 0; }
         ga[b] = a;
         // mode 1: V_b (kp1 x kp2 r3) = R_1b (kp1 x r1) U_b(1) (r1 x kp2 r3), scaled by the block scale
         GemmArgs c{};
         c.M = kp1; c.N = kp2 * r3; c.K = r1; c.nbatch = 1; c.acc = 0;
         c.A = static_cast<const T*>(p.Rp[0]) + (long long)B.off[0] * p.ldR[0]; c.lda = p.ldR[0]; c.sA = 0;
-        c.B = T1 + t1off; c.ldb = r1; c.sB = 0;
+        c.B = T1 + off; c.ldb = r1; c.sB = 0;
         c.C = Wm + (long long)B.off[2] * kp1 * kp2; c.ldc = kp1; c.sC = 0;
         c.alpha = B.scale; c.beta = 0.0;
-        if (r1 == 0 || r2 == 0 || r3 == 0) { c.M = 0; }
+        if (empty) c.M = 0;
         ga[TPCG_MAX_BLOCKS + b] = c;
-        t1off += (long long)r1 * kp2 * r3;
     }
+    if (b != 0) return;
+    const bool over = t1off > t1cap;   // workspace too small for these blocks: produce nothing, flag the plan
     // fused mode 3: Z (kp1 kp2 x kp3) = W (kp1 kp2 x k3) R_3^T
     GemmArgs z{};
-    z.M = kp1 * kp2; z.N = p.kp[2]; z.K = p.k[2]; z.nbatch = 1; z.acc = 0;
+    z.M = over ? 0 : kp1 * kp2; z.N = p.kp[2]; z.K = p.k[2]; z.nbatch = 1; z.acc = 0;
     z.A = Wm; z.lda = (long long)kp1 * kp2; z.sA = 0;
     z.B = p.Rp[2]; z.ldb = p.ldR[2]; z.sB = 0;
     z.C = Zout;
     z.ldc = (long long)kp1 * kp2; z.sC = 0;
     z.alpha = 1.0; z.beta = 0.0;
     ga[2 * TPCG_MAX_BLOCKS] = z;
-    counts[0] = p.nblk;
+    counts[0] = over ? 0 : p.nblk;
     if (prof) {
         const double e = sizeof(T);
         const double M3 = (double)kp1 * kp2, K3 = p.k[2], N3 = p.kp[2];
         prof[2 * PK_ZGEMM] += 2.0 * M3 * N3 * K3;
         prof[2 * PK_ZGEMM + 1] += e * (M3 * K3 + N3 * K3 + M3 * N3);
         double fb = 0;
-        for (int b = 0; b < p.nblk; ++b) {
-            const BlockDesc& B = d->blk[b];
-            fb += 2.0 * B.r[0] * kp2 * B.r[2] * B.r[1] + 2.0 * kp1 * kp2 * B.r[2] * B.r[0];
+        for (int q = 0; q < p.nblk; ++q) {
+            const BlockDesc& D = d->blk[q];
+            fb += 2.0 * D.r[0] * kp2 * D.r[2] * D.r[1] + 2.0 * kp1 * kp2 * D.r[2] * D.r[0];
         }
         prof[2 * PK_ZBLK] += fb;
     }
-    if (t1off > t1cap) {   // workspace too small for these blocks: produce nothing, flag the plan
+    if (over) {
         p.status = 1;
-        counts[0] = 0;
-        ga[2 * TPCG_MAX_BLOCKS].M = 0;
         for (int t = 0; t < 3; ++t) p.zdim[t] = 0;
     }
     *plan = p;
@@ -237,16 +257,12 @@ __global__ void __launch_bounds__(1024) qr_kernel(const RoundPlan* __restrict__ 
 //   m = 1: G = sum_i3 Z_i3^T Z_i3   (TN, slices i3 grouped)
 //   m = 2: G = Zmat^T Zmat          (TN, K = d1 d2 split)
 // --------------------------------------------------------------------------------------------------
+// Thread g plans partial g; d1, d2, d3: the working tensor's sizes (a single thread took 8 us to write 64 partials)
 template <typename T>
-__device__ void plan_gram(RoundPlan& p, GemmArgs* ga, const T* Zc, T* Part, int m, int nsplit_max, int min_k,
-                          int* counts, double* prof) {
-    const int d1 = p.zdim[0], d2 = p.zdim[1], d3 = p.zdim[2];
-    const int M = p.zdim[m];
-    int total = (m == 0) ? d2 * d3 : (m == 1 ? d3 : d1 * d2);
-    if (prof) {
-        prof[2 * PK_GRAM] += 2.0 * M * M * ((double)d1 * d2 * d3 / (M > 0 ? M : 1));
-        prof[2 * PK_GRAM + 1] += sizeof(T) * ((double)d1 * d2 * d3 + (double)M * M);
-    }
+__device__ void plan_gram(RoundPlan& p, GemmArgs* ga, const T* Zc, T* Part, int m, int d1, int d2, int d3, int nsplit_max,
+                          int min_k, int* counts, double* prof) {
+    const int M = m == 0 ? d1 : (m == 1 ? d2 : d3);
+    const int total = (m == 0) ? d2 * d3 : (m == 1 ? d3 : d1 * d2);
     int ns = total < nsplit_max ? total : nsplit_max;
     if (min_k > 0) {   // at least min_k of the reduction per group: fewer, longer groups (less partial traffic)
         const long long ktot = (long long)total * (m == 1 ? d1 : 1);
@@ -255,16 +271,14 @@ __device__ void plan_gram(RoundPlan& p, GemmArgs* ga, const T* Zc, T* Part, int 
     }
     if (ns < 1) ns = 1;
     if (M == 0 || total == 0) ns = 0;
-    const int chunk = ns ? (total + ns - 1) / ns : 0;
-    int used = 0;
-    for (int g = 0; g < ns; ++g) {
-        const int lo = g * chunk;
-        int hi = lo + chunk;
-        if (hi > total) hi = total;
-        if (lo >= hi) break;
+    const int chunk = ns ? (total + ns - 1) / ns : 1;
+    const int used = ns ? (total + chunk - 1) / chunk : 0;   // groups that begin before the end
+    const int g = threadIdx.x;
+    if (g < used) {
+        const int lo = g * chunk, hi = lo + chunk < total ? lo + chunk : total;
         GemmArgs a{};
         a.M = M; a.N = M; a.alpha = 1.0; a.beta = 0.0; a.sym = 1;
-        a.C = Part + (long long)used * M * M; a.ldc = M; a.sC = 0;
+        a.C = Part + (long long)g * M * M; a.ldc = M; a.sC = 0;
         if (m == 0) {
             a.K = hi - lo; a.nbatch = 1; a.acc = 0;
             a.A = Zc + (long long)lo * d1; a.lda = d1; a.sA = 0;
@@ -278,7 +292,12 @@ __device__ void plan_gram(RoundPlan& p, GemmArgs* ga, const T* Zc, T* Part, int 
             a.A = Zc + lo; a.lda = (long long)d1 * d2; a.sA = 0;
             a.B = Zc + lo; a.ldb = (long long)d1 * d2; a.sB = 0;
         }
-        ga[used++] = a;
+        ga[g] = a;
+    }
+    if (g != 0) return;
+    if (prof) {
+        prof[2 * PK_GRAM] += 2.0 * M * M * ((double)d1 * d2 * d3 / (M > 0 ? M : 1));
+        prof[2 * PK_GRAM + 1] += sizeof(T) * ((double)d1 * d2 * d3 + (double)M * M);
     }
     p.nsplit = used;
     p.gm = m;
@@ -287,31 +306,41 @@ __device__ void plan_gram(RoundPlan& p, GemmArgs* ga, const T* Zc, T* Part, int 
     p.rr = 0;
     counts[0] = used;
     counts[1] = M;
-    counts[2] = M;
 }
 
 // G = the sum of the partial Grams in their order, from their lower triangles (the GEMM need not compute the others);
-// M and the number of partials read from the device
+// M and the number of partials read from the device.
 template <typename T>
 __global__ void __launch_bounds__(256) gram_reduce_kernel(const T* __restrict__ P, const int* __restrict__ counts,
                                                           T* __restrict__ G) {
-    const int cnt = counts[0], M = counts[1];
-    const long long MM = (long long)M * M;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < MM; e += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(e % M), j = (int)(e / M);
-        if (i < j) continue;
+    // FP64: four lanes an entry, for a chain of additions (64 cycles each) a quarter as long.  FP32 keeps the order.
+    constexpr int L = sizeof(T) == 8 ? 4 : 1;
+    const int cnt = counts[0], M = counts[1], per = (cnt + L - 1) / L;
+    const long long MM = (long long)M * M, all = (MM * L + 31) & ~31LL;
+    for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < all; x += (long long)gridDim.x * blockDim.x) {
+        const long long e = x / L;
+        const int l = (int)(x % L), i = (int)(e % M), j = (int)(e / M);
+        const bool on = e < MM && i >= j;
         T s = T(0);
+        if (on) {
 #pragma unroll 16
-        for (int g = 0; g < cnt; ++g) s += P[g * MM + e];
-        G[e] = s;
-        G[j + (long long)i * M] = s;
+            for (int g = l * per; g < min(cnt, (l + 1) * per); ++g) s += P[g * MM + e];
+        }
+        if constexpr (L == 4) {
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+        }
+        if (on && l == 0) {
+            G[e] = s;
+            G[j + (long long)i * M] = s;
+        }
     }
 }
 
 template <typename T>
-__global__ void plan_gram_kernel(RoundPlan* plan, GemmArgs* ga, const T* Zc, T* Part, int m, int nsplit_max,
-                                 int min_k, int* counts, double* prof) {
-    if (threadIdx.x == 0) plan_gram<T>(*plan, ga, Zc, Part, m, nsplit_max, min_k, counts, prof);
+__global__ void __launch_bounds__(PLAN_THREADS) plan_gram_kernel(RoundPlan* plan, GemmArgs* ga, const T* Zc, T* Part, int m,
+                                                                 int nsplit_max, int min_k, int* counts, double* prof) {
+    plan_gram<T>(*plan, ga, Zc, Part, m, plan->zdim[0], plan->zdim[1], plan->zdim[2], nsplit_max, min_k, counts, prof);
 }
 
 // --------------------------------------------------------------------------------------------------
@@ -343,13 +372,17 @@ __device__ void plan_projection(RoundPlan& p, GemmArgs* ga, const void* S, long 
 // tensor's mode m shrinks to s_m, and for m < 2 the Gram of mode m + 1 of the projected tensor is planned into
 // gg (a separate argument range: the projection's product runs first)
 template <typename T>
-__global__ void plan_proj_kernel(RoundPlan* plan, GemmArgs* gp, const T* S, const T* Zc, T* Znext, int m,
+__global__ void __launch_bounds__(PLAN_THREADS) plan_proj_kernel(RoundPlan* plan, GemmArgs* gp, const T* S, const T* Zc, T* Znext, int m,
                                  GemmArgs* gg, T* Part, int nsplit_max, int min_k, int* counts, double* prof) {
-    if (threadIdx.x != 0) return;
     RoundPlan& p = *plan;
-    plan_projection(p, gp, S, p.n, Zc, Znext, m, p.s[m]);
-    p.zdim[m] = p.s[m];
-    if (m < 2) plan_gram<T>(p, gg, Znext, Part, m + 1, nsplit_max, min_k, counts, prof);
+    const int s = p.s[m];
+    const int d1 = m == 0 ? s : p.zdim[0], d2 = m == 1 ? s : p.zdim[1], d3 = m == 2 ? s : p.zdim[2];
+    __syncthreads();   // every thread has read the sizes
+    if (threadIdx.x == 0) {
+        plan_projection(p, gp, S, p.n, Zc, Znext, m, s);
+        p.zdim[m] = s;
+    }
+    if (m < 2) plan_gram<T>(p, gg, Znext, Part, m + 1, d1, d2, d3, nsplit_max, min_k, counts, prof);
 }
 
 // --------------------------------------------------------------------------------------------------
@@ -599,7 +632,7 @@ int round_stage12(tpcg_ctx c, tucker_t* y, double eps, const double* eps_dev, in
     GemmArgs* ga = c->gargs;
     int* counts = reinterpret_cast<int*>(c->scal + 200);   // 8 ints of scratch in the scalar area
     T* Z0 = static_cast<T*>(c->Z0);
-    plan_round_kernel<T><<<1, 32, 0, st>>>(static_cast<const TuckerDesc*>(y->desc), c->plan, ga, n, rc, eps, eps_dev,
+    plan_round_kernel<T><<<1, PLAN_THREADS, 0, st>>>(static_cast<const TuckerDesc*>(y->desc), c->plan, ga, n, rc, eps, eps_dev,
                                            c->Rq[0], c->Rq[1], c->Rq[2], y->U[0], y->U[1], y->U[2],
                                            static_cast<T*>(c->T1), static_cast<T*>(c->Wm), counts,
                                            (long long)c->max_cols * c->n * c->rank_cap, prof_dev(), strict_mode, Z0);
@@ -653,7 +686,7 @@ int round_stage34(tpcg_ctx c, tucker_t* y, double* info_dev, cudaStream_t st) {
     T* Zn = Z1;
     const int min_k = gram_min_k();
     GemmArgs* gproj = ga + MAX_SPLIT;   // projection arguments, apart from the next Gram's
-    plan_gram_kernel<T><<<1, 32, 0, st>>>(c->plan, ga, Zc, static_cast<T*>(c->Part), 0, MAX_SPLIT, min_k, counts,
+    plan_gram_kernel<T><<<1, PLAN_THREADS, 0, st>>>(c->plan, ga, Zc, static_cast<T*>(c->Part), 0, MAX_SPLIT, min_k, counts,
                                           prof_dev());
     TPCG_CHECK_LAUNCH();
     for (int m = 0; m < 3; ++m) {
@@ -662,7 +695,7 @@ int round_stage34(tpcg_ctx c, tucker_t* y, double* info_dev, cudaStream_t st) {
             TPCG_TRY((launch_gemm<T, false, true>(ga, counts, MAX_SPLIT, 1, n, n, st, true)));
         else
             TPCG_TRY((launch_gemm<T, true, false>(ga, counts, MAX_SPLIT, 1, n, n, st, true)));
-        gram_reduce_kernel<T><<<std::min((n * n + 255) / 256, 2 * sm_count()), 256, 0, st>>>(
+        gram_reduce_kernel<T><<<std::min((n * n + 63) / 64, 4 * sm_count()), 256, 0, st>>>(
             static_cast<const T*>(c->Part), counts, static_cast<T*>(c->Gm));
         TPCG_CHECK_LAUNCH();
         prof_end(PK_GRAM, st);
@@ -696,7 +729,7 @@ int round_stage34(tpcg_ctx c, tucker_t* y, double* info_dev, cudaStream_t st) {
         }
         prof_end(PK_EIG, st);
         prof_begin(PK_PROJ, st);
-        plan_proj_kernel<T><<<1, 32, 0, st>>>(c->plan, gproj, static_cast<const T*>(c->S[m]), Zc, Zn, m, ga,
+        plan_proj_kernel<T><<<1, PLAN_THREADS, 0, st>>>(c->plan, gproj, static_cast<const T*>(c->S[m]), Zc, Zn, m, ga,
                                               static_cast<T*>(c->Part), MAX_SPLIT, min_k, counts, prof_dev());
         TPCG_CHECK_LAUNCH();
         if (m == 0)
