@@ -6,6 +6,8 @@
 #include <mutex>
 #include <string>
 
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 #include "gemm.cuh"
 #include "kernels.cuh"
@@ -358,23 +360,52 @@ __global__ void plan_dot_kernel(const TuckerDesc* __restrict__ xd, const T* X0, 
     counts[0] = 3;
 }
 
+// *out = vec(G_x) . vec(Ta).  A cluster of DF_C CTAs: FP64 additions come at two a cycle and SM, and one SM took 25 us for the
+// 200,000 entries of a core of rank 58.  FP32 cores: every product as its rounded value and its exact error, summed in
+// pairs of floats (48 bits), which costs a twentieth of converting to FP64; the partial sums of the threads are added
+// in FP64, in a fixed order.
+constexpr int DF_C = 8, DF_T = 512;
+
 template <typename T>
-__global__ void dot_finish_kernel(const TuckerDesc* __restrict__ xd, const T* Ta, double* out, const int* bad) {
-    __shared__ double red[32];
-    if (*bad) {
-        if (threadIdx.x == 0) *out = nan("");
+__global__ void __cluster_dims__(DF_C, 1, 1) __launch_bounds__(DF_T)
+    dot_finish_kernel(const TuckerDesc* __restrict__ xd, const T* Ta, double* out, const int* bad) {
+    namespace cgx = cooperative_groups;
+    cgx::cluster_group cluster = cgx::this_cluster();
+    __shared__ double red[DF_T / 32], part[DF_C];
+    const int tid = threadIdx.x, rank = (int)cluster.block_rank();
+    if (*bad) {   // the whole cluster
+        if (rank == 0 && tid == 0) *out = nan("");
         return;
     }
     const long long tot = (long long)xd->rank[0] * xd->rank[1] * xd->rank[2];
     const T* Gx = static_cast<const T*>(xd->blk[0].core);
     double s = 0.0;
-    for (long long e = threadIdx.x; e < tot; e += blockDim.x) s += (double)Gx[e] * (double)Ta[e];
+    if constexpr (sizeof(T) == 8) {
+#pragma unroll 4
+        for (long long e = rank * DF_T + tid; e < tot; e += DF_C * DF_T) s = fma(Gx[e], Ta[e], s);
+    } else {
+        float hi = 0.f, lo = 0.f;
+#pragma unroll 4
+        for (long long e = rank * DF_T + tid; e < tot; e += DF_C * DF_T) {
+            const float x = Gx[e], y = Ta[e], p = __fmul_rn(x, y), pe = __fmaf_rn(x, y, -p);
+            const float t = __fadd_rn(hi, p), z = __fsub_rn(t, hi);   // t + err = hi + p exactly
+            lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(p, z)), pe));
+            hi = t;
+        }
+        s = (double)hi + (double)lo;
+    }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    if ((tid & 31) == 0) red[tid >> 5] = s;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
         double v = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[w];
+        for (int w = 0; w < DF_T / 32; ++w) v += red[w];
+        cluster.map_shared_rank(part, 0)[rank] = v;
+    }
+    cluster.sync();
+    if (rank == 0 && tid == 0) {
+        double v = 0.0;
+        for (int r = 0; r < DF_C; ++r) v += part[r];
         *out = v * xd->blk[0].scale;
     }
 }
@@ -398,7 +429,7 @@ int dot_impl(tpcg_ctx c, const tucker_t* x, const tucker_t* y, double* out_dev, 
     TPCG_TRY((launch_gemm<T, false, false>(ga + 3, nullptr, 1, 1, rc, rc * rc, st)));
     TPCG_TRY((launch_gemm<T, false, true>(ga + 4, nullptr, 1, rc, rc, rc, st)));
     TPCG_TRY((launch_gemm<T, false, true>(ga + 5, nullptr, 1, 1, rc * rc, rc, st)));
-    dot_finish_kernel<T><<<1, 1024, 0, st>>>(static_cast<const TuckerDesc*>(x->desc), Ta, out_dev, counts + 1);
+    dot_finish_kernel<T><<<DF_C, DF_T, 0, st>>>(static_cast<const TuckerDesc*>(x->desc), Ta, out_dev, counts + 1);
     TPCG_CHECK_LAUNCH();
     prof_end(PK_DOT, st);
     return TPCG_OK;
@@ -513,7 +544,7 @@ int dot_static_impl(const tucker_t* x, const tucker_t* y, double* out_dev, cudaS
     TPCG_TRY((launch_gemm<T, false, false>(ga + 3, nullptr, 1, 1, rc, rc * rc, st)));
     TPCG_TRY((launch_gemm<T, false, true>(ga + 4, nullptr, 1, rc, rc, rc, st)));
     TPCG_TRY((launch_gemm<T, false, true>(ga + 5, nullptr, 1, 1, rc * rc, rc, st)));
-    dot_finish_kernel<T><<<1, 1024, 0, st>>>(static_cast<const TuckerDesc*>(x->desc), Ta, out_dev, counts + 1);
+    dot_finish_kernel<T><<<DF_C, DF_T, 0, st>>>(static_cast<const TuckerDesc*>(x->desc), Ta, out_dev, counts + 1);
     TPCG_CHECK_LAUNCH();
     return TPCG_OK;
 }
