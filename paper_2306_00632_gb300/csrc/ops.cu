@@ -388,11 +388,15 @@ __global__ void __cluster_dims__(DF_C, 1, 1) __launch_bounds__(DF_T)
 #pragma unroll 4
         for (long long e = rank * DF_T + tid; e < tot; e += DF_C * DF_T) {
             const float x = Gx[e], y = Ta[e], p = __fmul_rn(x, y), pe = __fmaf_rn(x, y, -p);
+            if (!(fabsf(p) > 1e-28f && fabsf(p) < 1e30f)) {   // below, pe is inexact; above, a sum may overflow (or NaN)
+                if (p != 0.f || (x != 0.f && y != 0.f)) s = fma((double)x, (double)y, s);
+                continue;
+            }
             const float t = __fadd_rn(hi, p), z = __fsub_rn(t, hi);   // t + err = hi + p exactly
             lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(p, z)), pe));
             hi = t;
         }
-        s = (double)hi + (double)lo;
+        s += (double)hi + (double)lo;
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if ((tid & 31) == 0) red[tid >> 5] = s;

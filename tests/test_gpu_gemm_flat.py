@@ -70,3 +70,17 @@ def test_dot(api, dtype, n, rx, ry):
     u = 2.0 ** -24 if dtype else 2.0 ** -53
     scale = np.linalg.norm(X[0]) * np.linalg.norm(Y[0])
     assert abs(got - want) <= 10 * u * np.sqrt(n) * scale * max(rx + ry)
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+@pytest.mark.parametrize("sx,sy", [(1e-15, 1e-17), (1e-24, 1e-20), (1e20, 1e21), (1e25, 1e-25)])
+def test_dot_keeps_products_outside_fp32s_range(api, dtype, sx, sy):
+    n = 33
+    X, Y = _input(n, (9, 8, 7), 1), _input(n, (6, 9, 5), 2)
+    ctx = api.Ctx(n, 2 * n, n, dtype)
+    x = api.Tucker.from_numpy(X[0] * sx, X[1], dtype=dtype)
+    y = api.Tucker.from_numpy(Y[0] * sy, Y[1], dtype=dtype)
+    got = float(api.tucker_dot(ctx, x, y)) / sx / sy
+    want = float(np.sum(tucker.full(X) * tucker.full(Y)))
+    u = 2.0 ** -24 if dtype else 2.0 ** -53
+    assert abs(got - want) <= 10 * u * np.sqrt(n) * np.linalg.norm(X[0]) * np.linalg.norm(Y[0]) * 9
