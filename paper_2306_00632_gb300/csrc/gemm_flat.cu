@@ -188,6 +188,9 @@ int launch_gemm64(const GemmArgs* args, const int* count_dev, int ngroups, int b
 // without bank conflicts.  8 x 8 outputs are what the shared memory can feed (four 16-byte loads for 64 FMAs; 8 x 4 needs
 // three for 32); 8 x 4 where a product has no more than a few 64 x 64 tiles.  Operands are copied by cp.async through
 // GCP_STAGES stages, 16 bytes at a time where the layout and the alignment allow, and the last K-step stops at K.
+// FMAs are paired (two rows an instruction, same rounding): the FP32 units take them at the same rate, but half the issue
+// slots are left for the loads.  Truncated product n = 512 10.7 -> 10.2 ms (its largest contraction, 204 GFLOP, 3.9 ms: 52
+// TFLOP/s), n = 128 983 -> 950 us, mixed solve n = 128 186 -> 180 ms.
 // ------------------------------------------------------------------------------------------------------------
 __device__ __forceinline__ void cp_async16(float* dst, const float* src, int bytes) {
     const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
@@ -246,11 +249,11 @@ __global__ void __launch_bounds__(G32<TM, TN, CPT>::NT, G32<TM, TN, CPT>::MINB)
         const GfTile tl = gf_find<TM, TN>(args, pre, ng, t);
         const GemmArgs a = args[tl.g];
         const int M = a.M, N = a.N, K = a.K, m0 = tl.m0, n0 = tl.n0;
-        float acc[8][CPT];
+        float2 acc[4][CPT];   // rows 2 i and 2 i + 1 of the eight
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-            for (int j = 0; j < CPT; ++j) acc[i][j] = 0.f;
+            for (int j = 0; j < CPT; ++j) acc[i][j] = make_float2(0.f, 0.f);
         const int nb = a.acc ? a.nbatch : 1;
         const int nk = (K + GF_BK - 1) / GF_BK;
         for (int b = 0; b < nb; ++b) {
@@ -281,22 +284,24 @@ __global__ void __launch_bounds__(G32<TM, TN, CPT>::NT, G32<TM, TN, CPT>::MINB)
                 const float* Ac = As + cur * C32::AS + 4 * tx;
                 const float* Bc = Bs + cur * C32::BS + 4 * ty;
                 const int kn = K - kt * GF_BK;
-#pragma unroll
+#pragma unroll 1   // (unrolled further, the loads ahead do not fit in the registers)
                 for (int k4 = 0; k4 < GF_BK; k4 += 4) {
                     if (k4 >= kn) break;   // (rows past K are zero)
 #pragma unroll
                     for (int k1 = 0; k1 < 4; ++k1) {
                         const int kk = k4 + k1;
-                        float av[8], bv[CPT];
-                        *reinterpret_cast<float4*>(av) = *reinterpret_cast<const float4*>(Ac + kk * LDA);
-                        *reinterpret_cast<float4*>(av + 4) = *reinterpret_cast<const float4*>(Ac + kk * LDA + TM / 2);
+                        const float4 a0 = *reinterpret_cast<const float4*>(Ac + kk * LDA);
+                        const float4 a1 = *reinterpret_cast<const float4*>(Ac + kk * LDA + TM / 2);
+                        const float2 av[4] = {make_float2(a0.x, a0.y), make_float2(a0.z, a0.w), make_float2(a1.x, a1.y),
+                                              make_float2(a1.z, a1.w)};
+                        float bv[CPT];
                         *reinterpret_cast<float4*>(bv) = *reinterpret_cast<const float4*>(Bc + kk * LDB);
                         if constexpr (CPT == 8)
                             *reinterpret_cast<float4*>(bv + 4) = *reinterpret_cast<const float4*>(Bc + kk * LDB + TN / 2);
 #pragma unroll
-                        for (int i = 0; i < 8; ++i)
+                        for (int j = 0; j < CPT; ++j)
 #pragma unroll
-                            for (int j = 0; j < CPT; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+                            for (int i = 0; i < 4; ++i) acc[i][j] = __ffma2_rn(av[i], make_float2(bv[j], bv[j]), acc[i][j]);
                     }
                 }
                 cur = cur == GCP_STAGES - 1 ? 0 : cur + 1;
@@ -317,7 +322,10 @@ __global__ void __launch_bounds__(G32<TM, TN, CPT>::NT, G32<TM, TN, CPT>::MINB)
                 float* c = C + m + (long long)nI * a.ldc;
                 float v[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) v[i] = alpha * acc[4 * h + i][j];
+                for (int i = 0; i < 4; i += 2) {
+                    v[i] = alpha * acc[2 * h + i / 2][j].x;
+                    v[i + 1] = alpha * acc[2 * h + i / 2][j].y;
+                }
                 if (vc && m + 3 < M) {
                     *reinterpret_cast<float4*>(c) = make_float4(v[0], v[1], v[2], v[3]);
                 } else {
