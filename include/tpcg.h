@@ -324,7 +324,8 @@ void tpcg_elast_destroy(tpcg_elast e);
  *   eigenvectors (the pivoted Cholesky of G = Z Z^T is the column-pivoted QR of Z^T, the preconditioner of
  *   Drmac and Veselic's one-sided Jacobi SVD); 0 the two-sided cyclic Jacobi on G with accumulated rotations. */
 #define TPCG_OPT_EIG 3
-/*   TPCG_OPT_DST: how the preconditioner applies the sine block U_dft of App. B (Alg. 4): 1 (default) batched FFTs,
+/*   TPCG_OPT_DST: how the preconditioner applies the sine block U_dft of App. B (Alg. 4): 1 (default) for n1 <= 256 and
+ *   like ends two half-size dense products (its columns are even or odd about the middle), else batched FFTs,
  *   O(n1 log n1) per column, by Bluestein's chirp-z identity for any n1 <= 1024 (power-of-two FFTs of size
  *   >= 2 n1 - 1 in shared memory); 0 the dense n1 x n1 product with the stored sine matrix. */
 #define TPCG_OPT_DST 4

@@ -283,6 +283,7 @@ extern "C" int tpcg_ctx_create(int n, int max_cols, int rank_cap, int dtype, tpc
     TPCG_TRY(tc_prepare());
     TPCG_TRY(gemm32_prepare());
     TPCG_TRY(qr_prepare());
+    TPCG_TRY(fd_fold_prepare());
     (void)sm_count();
     tpcg_ctx c = new tpcg_ctx_s();
     c->lo = nullptr;
@@ -546,6 +547,12 @@ extern "C" int tpcg_problem_create(const tpcg_problem_arrays* a, tpcg_problem* o
         for (long long l = 0; l < n1; ++l) {
             const long long m = ((2 * j + sg.e) * (2 * l + sg.c) + sg.g) % (8 * sg.D);
             dst[l + j * n1] = sqrt(2.0) * sin(M_PI * (double)m / (4.0 * (double)sg.D));
+        }
+    pb->dst_sym = true;
+    for (long long j = 0; j < n1; ++j)
+        for (long long l = 0; l < n1; ++l) {
+            const double o = dst[n1 - 1 - l + j * n1];
+            if (fabs(dst[l + j * n1] - (j % 2 ? -o : o)) > 1e-13) pb->dst_sym = false;
         }
     std::vector<void*> owned;   // not used: problem buffers are tracked in the struct
     int s = TPCG_OK;

@@ -211,6 +211,7 @@ struct tpcg_problem_s {
     void* d_wtval;
     void* d_v2u2;        // n * n2
     void* d_dst;         // n1 x n1 sine matrix sqrt2 sin(j pi x_l)
+    bool dst_sym;        // its columns are alternately even and odd about the middle of the points
     void* d_chirp;       // chirp-z tables of the FFT sine transforms (complex pairs), null if n1 > 1024
     tpcg::ChirpInfo chirp;
     double* d_omega;     // RP

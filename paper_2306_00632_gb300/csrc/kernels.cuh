@@ -90,7 +90,48 @@ int chirp_tables(int n1, int p, int k0, int k1, ChirpInfo* info, std::vector<dou
 template <typename T>
 int launch_chirp(tpcg_problem pb, int kind, const TuckerDesc* sd, int mult, int rp_guard, int vcap, int maxcols,
                  const T* const* X, T* const* Y, int ldx, int ldy, cudaStream_t st);
-int dst_kind();   // TPCG_OPT_DST: 1 FFT sine transforms, 0 dense sine matrix
+int dst_kind();   // TPCG_OPT_DST: 1 half matrices or FFTs, 0 dense sine matrix
+// Alg. 4 with the two half matrices of a symmetric sine block (fd_fold.cu), for n1 up to FD_FOLD_MAX
+constexpr int FD_FOLD_MAX = 256;
+bool fd_fold_fits(tpcg_problem pb);
+template <typename T>
+int fd_fold(tpcg_problem pb, tpcg_ctx c, const tucker_t* s, tucker_t* v, const double* cw, double lmin, int* err,
+            cudaStream_t st);
+int fd_fold_prepare();   // shared-memory opt-in on the current device
+// descriptor of Alg. 4's output, written by one whole block: blocks (j, b) for every term j and input block b
+__device__ __forceinline__ void fd_desc(const TuckerDesc* __restrict__ sd, const double* __restrict__ omega, double lmin,
+                                        int RP, TuckerDesc* vd, int vcap, int* err, double* prof, int n, int n1, int n2, int p,
+                                        int elt) {
+    const int tid = threadIdx.x;   // a thread per block
+    if (prof && tid == 0) {   // algorithmic work of Alg. 4 per input column: W^T gather, sine transforms, R_P scalings, W scatter
+        const double cols = (double)sd->rank[0] + sd->rank[1] + sd->rank[2];
+        const double lg = n1 > 1 ? log2((double)n1) : 1.0;
+        prof[2 * PK_FD] += (1.0 + RP) * cols * (5.0 * n1 * lg + 4.0 * (p + 1) * n + 2.0 * (double)n * n2);
+        prof[2 * PK_FD + 1] += (double)elt * (double)n * cols * (2.0 + 2.0 * RP);
+    }
+    const int ns = sd->nblk;
+    bool ok = RP * ns <= TPCG_MAX_BLOCKS;
+    for (int t = 0; t < 3; ++t) ok = ok && (RP * sd->rank[t] <= vcap);
+    if (!ok) {
+        if (tid == 0) {
+            if (err) *err = 1;
+            vd->nblk = 0;
+            vd->rank[0] = vd->rank[1] = vd->rank[2] = 0;
+        }
+        return;
+    }
+    for (int e = tid; e < RP * ns; e += blockDim.x) {
+        const int j = e / ns, b = e % ns;
+        BlockDesc B = sd->blk[b];
+        for (int t = 0; t < 3; ++t) B.off[t] += j * sd->rank[t];
+        B.scale *= omega[j] / lmin;
+        vd->blk[e] = B;
+    }
+    if (tid == 0) {
+        vd->nblk = RP * ns;
+        for (int t = 0; t < 3; ++t) vd->rank[t] = RP * sd->rank[t];
+    }
+}
 
 int set_plain(tucker_t* t, int r1, int r2, int r3, cudaStream_t st);
 int set_zero(tucker_t* t, cudaStream_t st);

@@ -702,35 +702,7 @@ __global__ void fd_scatter_kernel(const TuckerDesc* __restrict__ sd, const T* A0
 __global__ void fd_desc_kernel(const TuckerDesc* __restrict__ sd, const double* __restrict__ omega, double lmin,
                                int RP, TuckerDesc* vd, int vcap, int* err, double* prof, int n, int n1, int n2, int p,
                                int elt) {
-    const int tid = threadIdx.x;   // a thread per block
-    if (prof && tid == 0) {   // algorithmic work of Alg. 4 per input column: W^T gather, sine transforms, R_P scalings, W scatter
-        const double cols = (double)sd->rank[0] + sd->rank[1] + sd->rank[2];
-        const double lg = n1 > 1 ? log2((double)n1) : 1.0;
-        prof[2 * PK_FD] += (1.0 + RP) * cols * (5.0 * n1 * lg + 4.0 * (p + 1) * n + 2.0 * (double)n * n2);
-        prof[2 * PK_FD + 1] += (double)elt * (double)n * cols * (2.0 + 2.0 * RP);
-    }
-    const int ns = sd->nblk;
-    bool ok = RP * ns <= TPCG_MAX_BLOCKS;
-    for (int t = 0; t < 3; ++t) ok = ok && (RP * sd->rank[t] <= vcap);
-    if (!ok) {
-        if (tid == 0) {
-            if (err) *err = 1;
-            vd->nblk = 0;
-            vd->rank[0] = vd->rank[1] = vd->rank[2] = 0;
-        }
-        return;
-    }
-    for (int e = tid; e < RP * ns; e += blockDim.x) {
-        const int j = e / ns, b = e % ns;
-        BlockDesc B = sd->blk[b];
-        for (int t = 0; t < 3; ++t) B.off[t] += j * sd->rank[t];
-        B.scale *= omega[j] / lmin;
-        vd->blk[e] = B;
-    }
-    if (tid == 0) {
-        vd->nblk = RP * ns;
-        for (int t = 0; t < 3; ++t) vd->rank[t] = RP * sd->rank[t];
-    }
+    fd_desc(sd, omega, lmin, RP, vd, vcap, err, prof, n, n1, n2, p, elt);
 }
 
 template <typename T>
@@ -748,6 +720,11 @@ int fd_impl(tpcg_problem pb, tpcg_ctx c, const tucker_t* s, tucker_t* v, cudaStr
         for (int q = 0; q < 4; ++q) buf[t][q] = static_cast<T*>(c->fd[t][q]);
     const TuckerDesc* sd = static_cast<const TuckerDesc*>(s->desc);
     prof_begin(PK_FD, st);
+    if (dst_kind() == 1 && fd_fold_fits(pb)) {
+        TPCG_TRY(fd_fold<T>(pb, c, s, v, cw, lmin, err, st));
+        prof_end(PK_FD, st);
+        return TPCG_OK;
+    }
     dim3 g1((n1 + 127) / 128, rc, 3);
     fd_gather_kernel<T><<<g1, 128, 0, st>>>(sd, static_cast<const T*>(s->U[0]), static_cast<const T*>(s->U[1]),
                                             static_cast<const T*>(s->U[2]), pb->d_wtrow, pb->d_wtcol,
