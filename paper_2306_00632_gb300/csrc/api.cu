@@ -284,6 +284,7 @@ extern "C" int tpcg_ctx_create(int n, int max_cols, int rank_cap, int dtype, tpc
     TPCG_TRY(gemm32_prepare());
     TPCG_TRY(qr_prepare());
     TPCG_TRY(fd_fold_prepare());
+    TPCG_TRY(dot_prepare());
     (void)sm_count();
     tpcg_ctx c = new tpcg_ctx_s();
     c->lo = nullptr;
@@ -731,11 +732,14 @@ extern "C" int tucker_axpby(double a, const double* a_dev, const tucker_t* x, do
 // Outside a stream capture, the public scalar products read both descriptors (16 bytes each, synchronising
 // the stream) and refuse a block tensor or a rank above the scratch limit with TPCG_E_INVALID.  Inside a
 // capture nothing can be read back: the kernels then write NaN for such inputs.
-static int check_dot_inputs(const tucker_t* x, const tucker_t* y, int max_rank, cudaStream_t st, const char* what) {
+// (staging: 32 bytes of pinned memory where the caller has them; copies to pageable memory wait one by one)
+static int check_dot_inputs(const tucker_t* x, const tucker_t* y, int max_rank, cudaStream_t st, const char* what,
+                            void* staging = nullptr) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     TPCG_CUDA(cudaStreamIsCapturing(st, &cs));
     if (cs != cudaStreamCaptureStatusNone) return TPCG_OK;
-    int h[2][4];
+    int local[2][4];
+    int(*h)[4] = staging ? static_cast<int(*)[4]>(staging) : local;
     TPCG_CUDA(cudaMemcpyAsync(h[0], x->desc, sizeof(h[0]), cudaMemcpyDeviceToHost, st));
     TPCG_CUDA(cudaMemcpyAsync(h[1], y->desc, sizeof(h[1]), cudaMemcpyDeviceToHost, st));
     TPCG_CUDA(cudaStreamSynchronize(st));
@@ -759,7 +763,7 @@ extern "C" int tucker_dot(tpcg_ctx c, const tucker_t* x, const tucker_t* y, doub
     if (!c || !out_dev) return TPCG_E_INVALID;
     TPCG_TRY(check_tensor(x, c->n, c->dtype, "tucker_dot x"));
     TPCG_TRY(check_tensor(y, c->n, c->dtype, "tucker_dot y"));
-    TPCG_TRY(check_dot_inputs(x, y, c->rank_cap, S(stream), "tucker_dot"));
+    TPCG_TRY(check_dot_inputs(x, y, c->rank_cap, S(stream), "tucker_dot", c->hstage));
     return by_dtype(c->dtype, [&](auto z) { return dot_impl<decltype(z)>(c, x, y, out_dev, S(stream)); });
 }
 

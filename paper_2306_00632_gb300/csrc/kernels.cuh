@@ -24,6 +24,7 @@ int round_mixed(tpcg_ctx c64, tpcg_ctx c32, tucker_t* y64, tucker_t* out32, doub
 // Householder QR Y_t = Q_t R_t of the modes with k_t < n (qr.cu), n <= QR_MAXN; W: n x n working copies, ld n everywhere
 constexpr int QR_MAXN = 512;
 int qr_prepare();
+int dot_prepare();
 template <typename T>
 int launch_qr(const RoundPlan* plan, int n, const T* const* Y, T* const* W, T* const* R, T* const* Q, cudaStream_t st);
 // whether a context of this size, rank cap and dtype reduces its large Grams by Rayleigh-Ritz

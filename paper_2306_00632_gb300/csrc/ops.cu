@@ -414,6 +414,133 @@ __global__ void __cluster_dims__(DF_C, 1, 1) __launch_bounds__(DF_T)
     }
 }
 
+// The whole product in one launch where the context's ranks are at most DS_R: a cluster of DS_C CTAs forms the W_t in every
+// CTA's shared memory (eight lanes an entry, lane l writes to the CTAs l and l + 8); then CTA c takes the slices j3 = c, c +
+// DS_C, ... of G_y:
+//   <x, y> = sum_j3 <G_y[:, :, j3] x_1 W_1 x_2 W_2, sum_i3 W_3[i3, j3] G_x[:, :, i3]>,
+// both r1 x r2, so that no tensor between the modes leaves the CTA.  Bound by latency.  Measured with the check of the inputs,
+// n = 32, FP64, against the six launches: rank 6 64 -> 20 us, rank 16 -> 30, rank 31 80 us (190 us with the contractions'
+// first kernels); FP32 62 -> 20 us at rank 6, 89 -> 45 us at rank 31.  Above rank 32 the work of 16 SMs would be the bound.
+constexpr int DS_C = 16, DS_T = 256, DS_R = 32;
+
+template <typename T>
+__global__ void __launch_bounds__(DS_T)
+    dot_small_kernel(const TuckerDesc* __restrict__ xd, const T* X0, const T* X1, const T* X2, const TuckerDesc* __restrict__ yd,
+                     const T* Y0, const T* Y1, const T* Y2, int n, int rc, double* out) {
+    namespace cgx = cooperative_groups;
+    cgx::cluster_group cluster = cgx::this_cluster();
+    __shared__ T W[3][DS_R * DS_R], Q[DS_R * DS_R], P[DS_R * DS_R];
+    __shared__ double red[DS_T / 32], part[DS_C];
+    const int tid = threadIdx.x, rank = (int)cluster.block_rank();
+    int r[3], s[3], E[3];
+    bool bad = xd->nblk != 1 || yd->nblk != 1;
+    for (int t = 0; t < 3; ++t) {
+        r[t] = xd->rank[t];
+        s[t] = yd->rank[t];
+        E[t] = r[t] * s[t];
+        bad = bad || r[t] > rc || s[t] > rc;
+    }
+    if (bad) {   // the whole cluster
+        if (rank == 0 && tid == 0) *out = nan("");
+        return;
+    }
+    cluster.sync();   // every CTA runs: remote writes may begin
+    const int l = tid & 7;
+    for (int base = 0; base < E[0] + E[1] + E[2]; base += DS_C * DS_T / 8) {   // the same trips in every lane
+        int e = base + (rank * DS_T + tid) / 8;
+        const bool on = e < E[0] + E[1] + E[2];
+        int t = 0;
+        while (on && e >= E[t]) e -= E[t++];
+        const int i = on ? e % r[t] : 0, j = on ? e / r[t] : 0;
+        T acc = T(0);
+        if (on) {
+            const T* x = (t == 0 ? X0 : (t == 1 ? X1 : X2)) + (long long)i * n;
+            const T* y = (t == 0 ? Y0 : (t == 1 ? Y1 : Y2)) + (long long)j * n;
+#pragma unroll 4
+            for (int k = l; k < n; k += 8) acc = fma(x[k], y[k], acc);
+        }
+        for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (on)
+            for (int c = l; c < DS_C; c += 8) cluster.map_shared_rank(&W[0][0], c)[t * DS_R * DS_R + i + j * DS_R] = acc;
+    }
+    cluster.sync();
+    const T* Gx = static_cast<const T*>(xd->blk[0].core);
+    const T* Gy = static_cast<const T*>(yd->blk[0].core);
+    const int r12 = r[0] * r[1], s12 = s[0] * s[1];
+    double sum = 0.0;
+    for (int j3 = rank; j3 < s[2]; j3 += DS_C) {
+        for (int e = tid; e < s12; e += DS_T) Q[e] = Gy[e + (long long)j3 * s12];
+        __syncthreads();
+        for (int e = tid; e < s[0] * r[1]; e += DS_T) {   // P = G_y[:, :, j3] W_2^T
+            const int i = e % s[0], b = e / s[0];
+            T acc = T(0);
+#pragma unroll 4
+            for (int a = 0; a < s[1]; ++a) acc = fma(Q[i + a * s[0]], W[1][b + a * DS_R], acc);
+            P[e] = acc;
+        }
+        __syncthreads();
+        for (int e = tid; e < r12; e += DS_T) {
+            const int i = e % r[0], b = e / r[0];
+            T u = T(0), v = T(0);
+#pragma unroll 4
+            for (int a = 0; a < s[0]; ++a) u = fma(W[0][i + a * DS_R], P[a + b * s[0]], u);
+#pragma unroll 4
+            for (int i3 = 0; i3 < r[2]; ++i3) v = fma(W[2][i3 + j3 * DS_R], Gx[e + (long long)i3 * r12], v);
+            sum = fma((double)u, (double)v, sum);
+        }
+        __syncthreads();   // before the next slice
+    }
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+    if ((tid & 31) == 0) red[tid >> 5] = sum;
+    __syncthreads();
+    if (tid == 0) {
+        double v = 0.0;
+        for (int w = 0; w < DS_T / 32; ++w) v += red[w];
+        cluster.map_shared_rank(part, 0)[rank] = v;
+    }
+    cluster.sync();
+    if (rank == 0 && tid == 0) {
+        double v = 0.0;
+        for (int c = 0; c < DS_C; ++c) v += part[c];
+        *out = v * xd->blk[0].scale * yd->blk[0].scale;
+    }
+}
+
+int dot_prepare() {   // clusters above 8 CTAs, once per device (takes driver locks: off the launch path)
+    static std::mutex mu;
+    static bool done[64] = {};
+    int dev = 0;
+    TPCG_CUDA(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) dev = 63;
+    std::lock_guard<std::mutex> lock(mu);
+    if (done[dev]) return TPCG_OK;
+    TPCG_CUDA(cudaFuncSetAttribute(dot_small_kernel<double>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    TPCG_CUDA(cudaFuncSetAttribute(dot_small_kernel<float>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    done[dev] = true;
+    return TPCG_OK;
+}
+
+template <typename T>
+static int launch_dot_small(const tucker_t* x, const tucker_t* y, int n, int rc, double* out_dev, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(DS_C);
+    cfg.blockDim = dim3(DS_T);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = DS_C;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    TPCG_CUDA(cudaLaunchKernelEx(&cfg, dot_small_kernel<T>, static_cast<const TuckerDesc*>(x->desc),
+                                 static_cast<const T*>(x->U[0]), static_cast<const T*>(x->U[1]), static_cast<const T*>(x->U[2]),
+                                 static_cast<const TuckerDesc*>(y->desc), static_cast<const T*>(y->U[0]),
+                                 static_cast<const T*>(y->U[1]), static_cast<const T*>(y->U[2]), n, rc, out_dev));
+    TPCG_CHECK_LAUNCH();
+    return TPCG_OK;
+}
+
 template <typename T>
 int dot_impl(tpcg_ctx c, const tucker_t* x, const tucker_t* y, double* out_dev, cudaStream_t st) {
     const int n = c->n, rc = c->rank_cap;
@@ -423,6 +550,11 @@ int dot_impl(tpcg_ctx c, const tucker_t* x, const tucker_t* y, double* out_dev, 
     T* Ta = static_cast<T*>(c->dotT);
     T* Tb = Ta + (long long)rc * rc * rc;
     prof_begin(PK_DOT, st);
+    if (rc <= DS_R) {
+        TPCG_TRY(launch_dot_small<T>(x, y, n, rc, out_dev, st));
+        prof_end(PK_DOT, st);
+        return TPCG_OK;
+    }
     plan_dot_kernel<T><<<1, 32, 0, st>>>(static_cast<const TuckerDesc*>(x->desc), static_cast<const T*>(x->U[0]),
                                          static_cast<const T*>(x->U[1]), static_cast<const T*>(x->U[2]),
                                          static_cast<const TuckerDesc*>(y->desc), static_cast<const T*>(y->U[0]),

@@ -84,3 +84,18 @@ def test_dot_keeps_products_outside_fp32s_range(api, dtype, sx, sy):
     want = float(np.sum(tucker.full(X) * tucker.full(Y)))
     u = 2.0 ** -24 if dtype else 2.0 ** -53
     assert abs(got - want) <= 10 * u * np.sqrt(n) * np.linalg.norm(X[0]) * np.linalg.norm(Y[0]) * 9
+
+
+@pytest.mark.parametrize("dtype", [0, 1])
+@pytest.mark.parametrize("n,rx,ry", [(2, (1, 1, 1), (1, 1, 1)), (9, (8, 9, 1), (1, 2, 9)), (32, (32, 32, 32), (32, 32, 32)),
+                                     (32, (31, 1, 17), (2, 32, 16)), (200, (17, 16, 32), (15, 9, 32)), (64, (5, 4, 3), (6, 5, 2))])
+def test_dot_in_one_launch(api, dtype, n, rx, ry):
+    X, Y = _input(n, rx, 3), _input(n, ry, 4)
+    cap = min(n, 32)   # the bound on the ranks that selects the single launch
+    ctx = api.Ctx(n, 2 * cap, cap, dtype)
+    x, y = (api.Tucker.from_numpy(*t, cap=max(rx + ry), dtype=dtype) for t in (X, Y))
+    want = float(np.sum(tucker.full(X) * tucker.full(Y)))
+    u = 2.0 ** -24 if dtype else 2.0 ** -53
+    bound = 10 * u * np.sqrt(n) * np.linalg.norm(X[0]) * np.linalg.norm(Y[0]) * max(rx + ry)
+    assert abs(float(api.tucker_dot(ctx, x, y)) - want) <= bound
+    assert abs(float(api.tucker_dot(ctx, y, x)) - want) <= bound
