@@ -91,8 +91,12 @@ __device__ __forceinline__ GfTile gf_find(const GemmArgs* __restrict__ args, con
 // quarter has work.  32 x 32 tiles, 128 threads: the lanes run along one side of the tile, the four warps share the other
 // side's rows in nearly equal parts (1 to 8 accumulators a thread, as many as there are rows); which side the lanes
 // take is the cheaper one of the two for the tile at hand.  With 64 x 64 tiles of 256 threads and 4 x 4 outputs each, a
-// product of 18 columns took 20 us, its padded tile's 65536 FMAs a K-step.
+// product of 18 columns took 20 us, its padded tile's 65536 FMAs a K-step.  The number of rows is a template parameter of
+// the K-step: with a test per FMA the switched-off ones took their cycles all the same (a Z formation of 97 columns 738 us,
+// now 617 us, 0.59 TFMA/s).  Where the tiles are fewer than the SMs, up to G64_PART CTAs share the rows of a tile (the 32 tiles
+// of a Z formation at n = 32 and 190 columns 54 -> 22 us; 8 CTAs a tile are no faster).
 // ------------------------------------------------------------------------------------------------------------
+constexpr int G64_PART = 4;   // CTAs that share the rows of a tile where the tiles are fewer than the SMs
 constexpr int G64_T = 32, G64_NT = 128, G64_LD = G64_T + 1, G64_Q = G64_T * GF_BK / G64_NT;
 
 // elements (i, k) of an operand: base[i si + k sk]; the threads run along whichever index is contiguous
@@ -114,19 +118,34 @@ __device__ __forceinline__ void g64_store(double* s, const double (&r)[G64_Q], l
     }
 }
 
+// a K-step of a warp with J rows.  J is known to the compiler: FMAs that a test at run time switches off take their cycles all
+// the same.
+template <int J>
+__device__ __forceinline__ void g64_step(double (&acc)[8], const double* X, const double* Y, int kn) {
+#pragma unroll 4
+    for (int kk = 0; kk < kn; ++kk) {
+        const double x = X[kk * G64_LD];
+#pragma unroll
+        for (int j = 0; j < J; ++j) acc[j] = fma(x, Y[kk * G64_LD + j], acc[j]);
+    }
+}
+
 __global__ void __launch_bounds__(G64_NT, 4) gemm64_kernel(const GemmArgs* __restrict__ args, const int* __restrict__ count_dev,
-                                                        int ngroups, int ta, int tb) {
+                                                        int ngroups, int ta, int tb, int sms) {
     __shared__ double As[GF_BK * G64_LD], Bs[GF_BK * G64_LD];
     __shared__ int pre[GF_MAXG], wsum[4];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int ng = count_dev ? min(*count_dev, ngroups) : ngroups;
     const int total = gf_list<G64_T, G64_T>(args, ng, pre, wsum);
-    for (int t = blockIdx.x; t < total; t += gridDim.x) {
-        const GfTile tl = gf_find<G64_T, G64_T>(args, pre, ng, t);
+    int part = 1;   // CTAs a tile
+    while (part < G64_PART && total * part <= sms) part *= 2;
+    for (int t = blockIdx.x; t < total * part; t += gridDim.x) {
+        const GfTile tl = gf_find<G64_T, G64_T>(args, pre, ng, t / part);
         const GemmArgs a = args[tl.g];
         const int mr = min(G64_T, a.M - tl.m0), nc = min(G64_T, a.N - tl.n0);
         const bool swap = mr < nc ? (mr + 3) / 4 < (nc + 3) / 4 : false;   // lanes along N, warps along M
-        const int cnt = swap ? mr : nc, per = (cnt + 3) / 4, c0 = warp * per, mine = max(0, min(per, cnt - c0));
+        const int cnt = swap ? mr : nc, per = (cnt + 4 * part - 1) / (4 * part);
+        const int c0 = (t % part * 4 + warp) * per, mine = max(0, min(per, cnt - c0));
         double acc[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) acc[j] = 0.0;
@@ -151,11 +170,16 @@ __global__ void __launch_bounds__(G64_NT, 4) gemm64_kernel(const GemmArgs* __res
                     g64_fetch(rb, B + (k0 + GF_BK) * bk, bn, bk, nc, a.K - k0 - GF_BK, tid);
                 }
                 const int kn = min(GF_BK, a.K - k0);
-                for (int kk = 0; kk < kn; ++kk) {
-                    const double x = X[kk * G64_LD];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        if (j < mine) acc[j] = fma(x, Y[kk * G64_LD + j], acc[j]);
+                switch (mine) {
+                    case 1: g64_step<1>(acc, X, Y, kn); break;
+                    case 2: g64_step<2>(acc, X, Y, kn); break;
+                    case 3: g64_step<3>(acc, X, Y, kn); break;
+                    case 4: g64_step<4>(acc, X, Y, kn); break;
+                    case 5: g64_step<5>(acc, X, Y, kn); break;
+                    case 6: g64_step<6>(acc, X, Y, kn); break;
+                    case 7: g64_step<7>(acc, X, Y, kn); break;
+                    case 8: g64_step<8>(acc, X, Y, kn); break;
+                    default: break;
                 }
             }
         }
@@ -177,8 +201,8 @@ int launch_gemm64(const GemmArgs* args, const int* count_dev, int ngroups, int b
                   cudaStream_t st) {
     const long long tiles = (long long)((Mmax + G64_T - 1) / G64_T) * ((Nmax + G64_T - 1) / G64_T) * ngroups * bmax;
     // four CTAs an SM: one is enough for the FP64 units, the others hide the loads of a K-step
-    const int grid = (int)std::min<long long>(tiles, 4LL * sm_count());
-    gemm64_kernel<<<grid, G64_NT, 0, st>>>(args, count_dev, ngroups, ta, tb);
+    const int grid = (int)std::min<long long>(tiles * G64_PART, 4LL * sm_count());
+    gemm64_kernel<<<grid, G64_NT, 0, st>>>(args, count_dev, ngroups, ta, tb, sm_count());
     TPCG_CHECK_LAUNCH();
     return TPCG_OK;
 }
