@@ -14,9 +14,9 @@
 // Four chains of additions an output: shorter chains round less (relative error in FP32 at n1 = 126 / 254: 1.1e-7 / 1.5e-7,
 // the FFTs 1.6e-7 / 1.7e-7; one chain 1.9e-7 / 2.8e-7).
 //
-// Measured, 12 terms on rank 44, against nine launches with FFTs: n = 128 FP64 242 -> 92 us (fwd 22, inv 65, out 8), FP32
-// 81 -> 27 us; rank 6, n = 32 FP64 80 -> 27 us; n = 256 FP64 328 -> 198 us, FP32 96 -> 40 us.  Loads one row after the other
-// (a trip to memory for the row's pointer, its column and the value) made it 98 us in place of 92 and, in FP32, 53 for 27.
+// Measured, 12 terms on rank 44, against nine launches with FFTs: n = 128 FP64 242 -> 76 us, FP32 81 -> 25 us; rank 6,
+// n = 32 FP64 80 -> 22 us; n = 256 FP64 328 -> 173 us, FP32 96 -> 36 us.  Loads one row after the other (a trip to memory for
+// the row's pointer, its column and the value) cost another 26 us in FP32.
 #include <math.h>
 
 #include <algorithm>
@@ -160,6 +160,35 @@ __global__ void __launch_bounds__(FF_FWD_T) fd_fold_fwd_kernel(const FdFold<T> a
     }
 }
 
+// Rows of one warp (the first PW of its FF_RW places in m): sums over the even and the odd sinusoids, stored to both halves
+template <typename T, int PW>
+__device__ __forceinline__ void ff_rows(const T* x, const T* m, int n1, int n1p, int l0, int H, bool in, T* __restrict__ A,
+                                        int cols, int col) {
+    T s[PW][2][4];
+#pragma unroll
+    for (int i = 0; i < PW; ++i)
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s[i][k & 1][k >> 1] = T(0);
+    for (int q = 0; q < n1p; q += 8) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const T xv = x[(q + k) * FF_TC];
+            const T* mq = m + (q + k) * 4 * FF_RW;
+#pragma unroll
+            for (int i = 0; i < PW; ++i) s[i][k & 1][k >> 1] = fma(mq[i], xv, s[i][k & 1][k >> 1]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < PW; ++i) {
+        const int l = l0 + i;
+        if (!in || l >= H) continue;
+        const T e = (s[i][0][0] + s[i][0][1]) + (s[i][0][2] + s[i][0][3]);
+        const T o = (s[i][1][0] + s[i][1][1]) + (s[i][1][2] + s[i][1][3]);
+        A[(long long)l * cols + col] = e + o;
+        if (l != n1 - 1 - l) A[(long long)(n1 - 1 - l) * cols + col] = e - o;
+    }
+}
+
 // A work item: FF_TC columns of one mode and 4 `pw` rows of the half (pw a warp).  pw is the one for which the SMs' largest
 // share of items costs least: small tensors get one row a warp and all SMs, large ones four, which halves the share of the
 // work that makes the scaled columns (a quarter of a row each).
@@ -191,43 +220,20 @@ __global__ void __launch_bounds__(FF_INV_T) fd_fold_inv_kernel(const FdFold<T> a
         const T* __restrict__ f = a.F[t] + (long long)j * a.n;
         __syncthreads();   // the previous item is done with x
 #pragma unroll 8
-        for (int e = tid; e < n1p * 4 * FF_RW; e += FF_INV_T) {   // (rows past pw are not read)
-            const int i = e % (4 * FF_RW), q = e / (4 * FF_RW), l = (w % per) * 4 * pw + i;
-            m[e] = q < n1 && i < 4 * pw && l < H ? a.dst[l + (long long)q * n1] : T(0);
+        for (int e = tid; e < n1p * 4 * FF_RW; e += FF_INV_T) {   // FF_RW places a warp, pw of them used
+            const int i = e % FF_RW, q = e / (4 * FF_RW), l = (w % per) * 4 * pw + e / FF_RW % 4 * pw + i;
+            m[e] = q < n1 && i < pw && l < H ? a.dst[l + (long long)q * n1] : T(0);
         }
 #pragma unroll 8
         for (int q = warp; q < n1p; q += FF_INV_T / 32) x[q * FF_TC + lane] = q < n1 ? f[q] * u[(long long)q * r] : T(0);
         __syncthreads();
-        T s[FF_RW][2][4];
-#pragma unroll
-        for (int i = 0; i < FF_RW; ++i)
-#pragma unroll
-            for (int k = 0; k < 8; ++k) s[i][k & 1][k >> 1] = T(0);
-        const int rows = min(pw, H - l0);   // (negative: none)
-        if (rows > 0) {
-            const T* mw = m + warp * pw;
-            for (int q = 0; q < n1p; q += 8) {
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const T xv = x[(q + k) * FF_TC + lane];
-                    const T* mq = mw + (q + k) * 4 * FF_RW;
-#pragma unroll
-                    for (int i = 0; i < FF_RW; ++i)
-                        if (i < rows) s[i][k & 1][k >> 1] = fma(mq[i], xv, s[i][k & 1][k >> 1]);
-                }
-            }
-        }
-        if (col < cols) {
-            T* __restrict__ A = a.A[t];
-#pragma unroll
-            for (int i = 0; i < FF_RW; ++i)
-                if (i < rows) {
-                    const int l = l0 + i;
-                    const T e = (s[i][0][0] + s[i][0][1]) + (s[i][0][2] + s[i][0][3]);
-                    const T o = (s[i][1][0] + s[i][1][1]) + (s[i][1][2] + s[i][1][3]);
-                    A[(long long)l * cols + col] = e + o;
-                    if (l != n1 - 1 - l) A[(long long)(n1 - 1 - l) * cols + col] = e - o;
-                }
+        const T *xl = x + lane, *mw = m + warp * FF_RW;
+        const bool in = col < cols;
+        switch (pw) {   // (a count known to the compiler: a test per multiply-add made five instructions of one)
+            case 1: ff_rows<T, 1>(xl, mw, n1, n1p, l0, H, in, a.A[t], cols, col); break;
+            case 2: ff_rows<T, 2>(xl, mw, n1, n1p, l0, H, in, a.A[t], cols, col); break;
+            case 3: ff_rows<T, 3>(xl, mw, n1, n1p, l0, H, in, a.A[t], cols, col); break;
+            default: ff_rows<T, FF_RW>(xl, mw, n1, n1p, l0, H, in, a.A[t], cols, col); break;
         }
     }
 }
