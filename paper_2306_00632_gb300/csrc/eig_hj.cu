@@ -13,7 +13,7 @@
 //     memory.  2 Ce - 1 rounds and the pairs inside the blocks make a sweep in which every pair meets once.  The
 //     cluster waits for itself once a round, not once a step.
 //
-// What bounds it: a chain of about rc steps a sweep (5 to 6 sweeps in FP64, 4 in FP32), each a dot product, its
+// What bounds it: a chain of about rc steps a sweep (5 to 7 sweeps), each a dot product, its
 // reduction, the rotation's parameters and the rotation.  In FP64 the arithmetic: an FP64 instruction of a warp takes
 // its quarter of the SM 64 cycles, dependent or not, so a step costs what one quarter issues (13 + 4 M / 32
 // instructions for one pair).  Hence one pair per quarter, on as many CTAs as the columns fill so; shears with three
@@ -45,6 +45,11 @@ template <typename T>
 __host__ __device__ constexpr T hj_tau() { return sizeof(T) == 8 ? T(1e-14) : T(5e-7); }
 template <typename T>
 __host__ __device__ constexpr T hj_last() { return sizeof(T) == 8 ? T(1e-8) : T(1.5e-3); }
+
+// The sweep after one that met a cosine above this is steered in FP32 (46 us in place of 75 us at order 97).  Below it the
+// products that FP32 leaves count: at 1e-3 most Grams took a sweep more (order 97: 550 us, 521 us at 2e-2, 554 us unsteered;
+// order 32 188 us, 187 us and 213 us; three Grams of order 64 in a sum 703, 690 and 779 us).
+constexpr float HJ_STEER = 2e-2f;
 
 // Shape of a launch: C CTAs, LPP lanes per pair of columns, RPL rows per lane (orders up to LPP RPL), BT pairs a CTA
 // takes at a time before another CTA joins.
@@ -118,24 +123,45 @@ __device__ __forceinline__ void hj_save(const T (&x)[RPL], T* a, int gl, int rpl
 // as the shears x -= u y, y += s x, x -= u y (three FMAs an element).  The angle needs no more than FP32: an error of
 // 1e-6 in it leaves 1e-6 of the product for the next sweep; s = 2 u / (1 + u^2) has the working precision, so that the
 // shears make an orthogonal matrix.
-template <typename T, int LPP, int RPL>
+//
+// STEER (FP64, the first sweeps): everything but the shears and s in FP32 as well, the dot product and the norms included.
+// Their error of 1e-6 |x| |y| stays for the sweeps that follow, and an FP64 step of 17 instructions at 32 rows becomes one of 8.
+template <typename T, int LPP, int RPL, bool STEER = false>
 __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, int rpl, T skip, T floor_g, int& big) {
     T g = T(0);
     if constexpr (hj_vec<T, LPP, RPL>) {
         const float2 g2 = __ffma2_rn(make_float2(x[2], x[3]), make_float2(y[2], y[3]),
                                      __fmul2_rn(make_float2(x[0], x[1]), make_float2(y[0], y[1])));
         g = g2.x + g2.y;
-    } else {
+    } else if constexpr (!STEER) {
 #pragma unroll
         for (int q = 0; q < RPL; ++q)
             if (q < rpl) g = fma(x[q], y[q], g);
     }
+    if constexpr (!STEER) {
 #pragma unroll
-    for (int o = LPP / 2; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+        for (int o = LPP / 2; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+    }
     float fa, fb, fg, fd;   // |x|^2, |y|^2, x . y, |y|^2 - |x|^2
     int off = 0;
     bool on;
-    if constexpr (sizeof(T) == 8) {   // by a power of two near the larger norm: nothing that counts leaves FP32's range
+    float g0 = 0.f, a0 = 0.f, b0 = 0.f;   // STEER: product and norms before the scaling
+    if constexpr (STEER) {
+#pragma unroll
+        for (int q = 0; q < RPL; ++q)
+            if (q < rpl) g0 = fmaf(hj_to_float(x[q], 0), hj_to_float(y[q], 0), g0);
+#pragma unroll
+        for (int o = LPP / 2; o > 0; o >>= 1) g0 += __shfl_xor_sync(0xffffffffu, g0, o);
+        a0 = hj_to_float(ax, 0);
+        b0 = hj_to_float(ay, 0);
+        const float sc = __int_as_float(0x7f000000 - (__float_as_int(fmaxf(a0, b0)) & 0x7f800000));   // larger norm to [1, 2)
+        fa = a0 * sc;
+        fb = b0 * sc;
+        fg = g0 * sc;
+        fd = fb - fa;
+        const int hs = __double2hiint(skip);
+        on = fa > 0.f && fb > 0.f && (__double2hiint(ax) > hs || __double2hiint(ay) > hs);
+    } else if constexpr (sizeof(T) == 8) {   // by a power of two near the larger norm: nothing that counts leaves FP32's range
         const int hx = __double2hiint(ax), hy = __double2hiint(ay), hs = __double2hiint(skip);
         off = (max(hx, hy) >> 20) - 1023;
         fa = hj_to_float(ax, off);
@@ -159,7 +185,11 @@ __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, 
     const float u = t * fmaf(w, fmaf(w, fmaf(w, fmaf(w, fmaf(w, -0.00342296f, 0.0151217f), -0.03403639f), 0.06147052f),
                              -0.12491905f), 0.49999894f);
     bool above, large;
-    if constexpr (sizeof(T) == 8) {
+    if constexpr (STEER) {
+        const float cs = ag * rsqrtf(fa) * rsqrtf(fb);
+        above = cs > 2e-6f;
+        large = cs > HJ_STEER;
+    } else if constexpr (sizeof(T) == 8) {
         const float rab = ab > 0.f ? ab * rsqrtf(ab) : 0.f;
         above = ag > (float)hj_tau<T>() * rab;
         large = ag > (float)hj_last<T>() * rab;
@@ -207,7 +237,10 @@ __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, 
                 }
         }
         const float tg = t * fg;   // the norms are exact again at the next sweep
-        if constexpr (sizeof(T) == 8) {
+        if constexpr (STEER) {
+            ax = hj_to_double(fmaxf(a0 - t * g0, 0.f));
+            ay = hj_to_double(fmaxf(b0 + t * g0, 0.f));
+        } else if constexpr (sizeof(T) == 8) {
             if (fabsf(tg) > 1e-30f) {
                 const double v = hj_to_double(tg, off);
                 ax -= v;
@@ -288,6 +321,7 @@ __global__ void __launch_bounds__(SH::NT, 1)
     __shared__ double s_piv[2][C], dg[NQ];           // their values; remaining diagonal of this CTA's columns
     __shared__ int dg0[NQ];                          // leading bits of what counts as noise there
     __shared__ float dgf[sizeof(T) == 4 ? ROWS : 1];
+    __shared__ double dga[sizeof(T) == 8 && RPL == 1 ? ROWS : 1];   // the whole remaining diagonal
     __shared__ short piv_of[ROWS];
     __shared__ int s_flags[2][C];
     __shared__ double s_red[32], s_rem, lam[ROWS], lsort[ROWS], disc[ROWS + 1];
@@ -353,7 +387,71 @@ __global__ void __launch_bounds__(SH::NT, 1)
     // ---- 1. pivoted Cholesky.  How the columns of L are spread over the cluster depends on their number: they wait in
     // shared memory (FP64) or in S (FP32)
     int rc = 0;
-    if constexpr (sizeof(T) == 8) {
+    if constexpr (sizeof(T) == 8 && RPL == 1) {
+        // Up to 32 rows every CTA factorises the whole Gram in its registers, row `lane` and columns warp + NW q (the columns
+        // spread over the cluster cost a barrier of the cluster a step, more than their FMAs)
+        constexpr int NW = NT / 32, NA = ROWS / NW;
+        double Ar[NA];
+#pragma unroll
+        for (int q = 0; q < NA; ++q) {
+            const int j = warp + NW * q;
+            Ar[q] = lane < M && j < M ? G[lane + (long long)j * M] * sc : 0.0;
+        }
+        const double d0 = lane < M ? G[lane + (long long)lane * M] * sc : -1.0;
+        // an entry below 8 u of what the Gram had there is rounding noise and no candidate
+        const int noise = __double2hiint(fmax(8 * 1.1102230246251565e-16 * d0, 1e-30));
+        if (warp == 0) dga[lane] = d0;
+        __syncthreads();
+        const float stop_rem = (float)(1e-10 * bus);
+        unsigned gone = 0;   // pivoted rows and columns
+        for (int k = 0; k < M; ++k) {
+            const double d = dga[lane];   // remaining diagonal, -1 once pivoted
+            const int hi = __double2hiint(d);
+            const int key = hi > noise ? hi : -1;
+            const int best = __reduce_max_sync(FULL, key);
+            const int piv = __ffs(__ballot_sync(FULL, key == best)) - 1;
+            float left = hi > 0 ? hj_to_float(d, 0) : 0.f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) left += __shfl_xor_sync(FULL, left, o);
+            if (best < 0 || !(left > stop_rem)) break;   // the same in every thread of the cluster
+            double* lk = lbuf[k & 1];
+            if (warp == piv % NW) {
+                double a = 0.0;
+#pragma unroll
+                for (int q = 0; q < NA; ++q) a = q == piv / NW ? Ar[q] : a;
+                a = gone >> lane & 1 ? 0.0 : a;
+                lk[lane] = a;
+                if (k % C == crank) cols[(k / C) * LD + lane] = a;
+            }
+            // A -= a a^T / d of the column a as it is; the scaling of L's column waits until it is read back
+            const double dp = __shfl_sync(FULL, d, piv);
+            const double r0 = hj_to_double(__fdividef(1.f, hj_to_float(dp, 0)));
+            const double er = fma(-dp, r0, 1.0), invd = fma(r0, fma(er, er, er), r0);
+            gone |= 1u << piv;
+            if (tid == 0) {
+                piv_of[k] = (short)piv;
+                lam[k] = dp;
+            }
+            __syncthreads();
+            const double li = -lk[lane] * invd;
+#pragma unroll
+            for (int q = 0; q < NA; ++q) {
+                const int j = warp + NW * q;
+                if (j >= M || (gone >> j & 1)) continue;
+                Ar[q] = fma(li, lk[j], Ar[q]);
+                if (lane == j) dga[j] = Ar[q];
+            }
+            if (tid == 0) dga[piv] = -1.0;
+            __syncthreads();
+            rc = k + 1;
+        }
+        if (warp == 0) {   // energy outside the columns of L
+            const double d = dga[lane];
+            const double t = hj_warp_sum(d > 0.0 ? d : 0.0);
+            if (lane == 0) s_rem = t * unscale;
+        }
+        cluster.sync();   // columns complete
+    } else if constexpr (sizeof(T) == 8) {
         // The columns of G are spread over the cluster, column j in CTA j mod C, and every step waits for the cluster
         // once.
         T* A = cols + 2 * BMAX * LD;                     // what other CTAs read; the own columns are in registers as well
@@ -567,6 +665,7 @@ __global__ void __launch_bounds__(SH::NT, 1)
     const T floor_g = sizeof(T) == 8 ? T(0) : T(1e-12f) * tr;   // FP32 products below this are noise of the factor
     auto column = [&](int set, int blk, int pos) -> T* { return cols + ((set * 2 + blk) * BMAX + pos) * LD; };
     T x[RPL], y[RPL];
+    bool steer = sizeof(T) == 8;
     for (int sweep = 0; sweep < max_sweeps && rc > 1; ++sweep) {
         ++nsweeps;
         int big = 0;   // a rotation that is not small
@@ -606,7 +705,8 @@ __global__ void __launch_bounds__(SH::NT, 1)
                 T ax = on ? nrm[set][blk][i] : T(0), ay = on ? nrm[set][blk][j] : T(0);
                 hj_load<T, LPP, RPL>(x, xp, gl, rpl);
                 hj_load<T, LPP, RPL>(y, yp, gl, rpl);
-                hj_pair<T, LPP, RPL>(x, y, ax, ay, rpl, skip, floor_g, big);
+                if (sizeof(T) == 8 && steer) hj_pair<T, LPP, RPL, sizeof(T) == 8>(x, y, ax, ay, rpl, skip, floor_g, big);
+                else hj_pair<T, LPP, RPL>(x, y, ax, ay, rpl, skip, floor_g, big);
                 if (on) {
                     hj_save<T, LPP, RPL>(x, xp, gl, rpl);
                     hj_save<T, LPP, RPL>(y, yp, gl, rpl);
@@ -629,7 +729,8 @@ __global__ void __launch_bounds__(SH::NT, 1)
                 if (wact) {
                     T ay = act ? nrm[set][1][j] : T(0);
                     hj_load<T, LPP, RPL>(y, yp, gl, rpl);
-                    hj_pair<T, LPP, RPL>(x, y, ax, ay, rpl, skip, floor_g, big);
+                    if (sizeof(T) == 8 && steer) hj_pair<T, LPP, RPL, sizeof(T) == 8>(x, y, ax, ay, rpl, skip, floor_g, big);
+                    else hj_pair<T, LPP, RPL>(x, y, ax, ay, rpl, skip, floor_g, big);
                     if (act) {
                         hj_save<T, LPP, RPL>(y, yp, gl, rpl);
                         if (gl == 0) nrm[set][1][j] = ay;
@@ -642,7 +743,8 @@ __global__ void __launch_bounds__(SH::NT, 1)
             }
             if (round == 2 * Ce - 2) {   // did this sweep rotate by more than a little? told to every CTA
                 const int any = __syncthreads_or(big);
-                if (tid < C && crank < Ce) cluster.map_shared_rank(&s_flags[sweep & 1][0], tid)[crank] = any;
+                const int tell = sizeof(T) == 8 && steer ? (any ? 3 : 1) : any;   // a steered sweep is never the last one
+                if (tid < C && crank < Ce) cluster.map_shared_rank(&s_flags[sweep & 1][0], tid)[crank] = tell;
             }
             if (Ce == 1) {
                 if (act) {
@@ -672,6 +774,7 @@ __global__ void __launch_bounds__(SH::NT, 1)
         int fl = 0;
         for (int r = 0; r < Ce; ++r) fl |= s_flags[sweep & 1][r];
         if (!fl) break;   // no rotation, or only small ones
+        steer = steer && (fl & 2);
     }
     // ---- 3. eigenvalues (exact squared norms) to CTA 0, decreasing order, truncation rule, normalised kept columns.
     // 2 Ce - 1 moves bring every block home, so player k is where the Cholesky put it.
