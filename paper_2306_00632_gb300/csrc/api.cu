@@ -4,8 +4,10 @@
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
+#include <sys/prctl.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <mutex>
 #include <string>
@@ -857,8 +859,33 @@ int tpcg::ensure_tensors(tpcg_ctx c, int count) {
 // sleeps.  Neither spinning in the driver (one core per waiting solver thread) nor a blocking-sync wait
 // (woken through the driver's interrupt path, slow once tens of solver threads wait at once) shares the host
 // cores as well when many solves run concurrently.
+//
+// With the default timer slack of 50 us a sleep of 10 or 20 us takes 60 to 70, and the GPU waits for the thread at every
+// decision of Alg. 2.  While at most FINE_WAITERS threads wait they sleep 10 us in earnest (slack 1 us, given back after the
+// wait): mixed solve n = 128 186.8 -> 182.6 ms, FP64 solve n = 32 112.6 -> 110.4 ms, for 20 ms of a core each.  More
+// threads would gain 1% and cost a core for every four of them.
+constexpr int FINE_WAITERS = 4;
+static std::atomic<int> g_waiters{0};
+struct Waiter {
+    const bool few = g_waiters.fetch_add(1, std::memory_order_relaxed) < FINE_WAITERS;
+    long slack = -1;   // the thread's own
+    std::chrono::microseconds nap() {
+        if (!few) return std::chrono::microseconds(20);
+        if (slack < 0) {
+            slack = prctl(PR_GET_TIMERSLACK, 0UL, 0UL, 0UL, 0UL);
+            if (slack > 0) prctl(PR_SET_TIMERSLACK, 1000UL, 0UL, 0UL, 0UL);
+        }
+        return std::chrono::microseconds(10);
+    }
+    ~Waiter() {
+        if (slack > 0) prctl(PR_SET_TIMERSLACK, (unsigned long)slack, 0UL, 0UL, 0UL);
+        g_waiters.fetch_sub(1, std::memory_order_relaxed);
+    }
+};
+
 int tpcg::host_wait(tpcg_ctx c, cudaStream_t s) {
     TPCG_CUDA(cudaEventRecord(c->sync_ev, s));
+    Waiter waiter;
     for (int it = 0;; ++it) {
         const cudaError_t e = cudaEventQuery(c->sync_ev);
         if (e == cudaSuccess) return TPCG_OK;
@@ -867,10 +894,11 @@ int tpcg::host_wait(tpcg_ctx c, cudaStream_t s) {
             set_error(std::string("host_wait: ") + cudaGetErrorString(e));
             return TPCG_E_CUDA;
         }
-        if (it < 16)
+        if (it < 16) {
             std::this_thread::yield();
-        else
-            std::this_thread::sleep_for(std::chrono::microseconds(20));
+        } else {
+            std::this_thread::sleep_for(waiter.nap());
+        }
     }
 }
 
