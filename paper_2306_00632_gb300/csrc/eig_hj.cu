@@ -19,7 +19,7 @@
 // instructions for one pair).  Hence one pair per quarter, on as many CTAs as the columns fill so; shears with three
 // FMAs an element; everything that only steers the iteration in FP32; and no rotation of pairs far below the budget.
 // Measured, FP64, a Gram of order 120 and full rank: 1.5 ms (16 CTAs), where the two-sided cyclic Jacobi on 8 CTAs that
-// this replaces took 18 ms at order 97; order 32: 0.22 ms against 0.8 ms.  FP32, where a step is latency and instructions
+// this replaces took 18 ms at order 97; order 32: 0.19 ms against 0.8 ms.  FP32, where a step is latency and instructions
 // (0.3 us with 16-byte accesses and paired FMAs, 0.45 us without): order 128 and rank 45 0.14 ms, where a ring of columns in
 // one CTA's registers with a barrier a step took 0.43 ms.
 #include <math.h>
