@@ -39,12 +39,26 @@ namespace cgx = cooperative_groups;
 
 // A pair is orthogonal once |a_p . a_q| <= tau |a_p| |a_q|.  FP32: the dot product itself resolves about 4e-7 at 128
 // rows.  FP64: at 2e-13 the truncated tensors were up to five times further from the 64-bit ones than at 1e-14, in
-// the same time.  A sweep whose rotations were all below `last` is the last one: the convergence is quadratic, so the next
-// would only meet products near last^2.
+// the same time.
+//
+// A rotation of p and q by theta gives the product (p, r) the part sin(theta) (q, r), so what a sweep leaves behind is at
+// most its largest cosine times its largest sine.  It is the last one when its cosines were all below `last` and its
+// |u| = |tan(theta / 2)| all below `turn`: 2 turn last = 2e-14 (FP64) and 9e-6 (FP32) may stay.  The cosines alone say
+// nothing where norms nearly coincide: there a cosine of 1e-10 turns by 45 degrees (with that rule the kept vectors of triples of
+// singular values 1e-9 apart were orthonormal to 2e-10 in place of 1e-14, in FP32 to 4e-4).  FP32: wide turns do not
+// count in a sweep whose cosines were all below `rest`, which may stay; pairs of equal norm would go on turning on
+// the rounding of their products.
 template <typename T>
 __host__ __device__ constexpr T hj_tau() { return sizeof(T) == 8 ? T(1e-14) : T(5e-7); }
 template <typename T>
 __host__ __device__ constexpr T hj_last() { return sizeof(T) == 8 ? T(1e-8) : T(1.5e-3); }
+template <typename T>
+__host__ __device__ constexpr float hj_turn() { return sizeof(T) == 8 ? 1e-6f : 3e-3f; }
+constexpr float HJ_REST = 3e-6f;
+
+// what a sweep met: a large cosine (or, FP64, a wide turn); FP32: a wide turn, a cosine above HJ_REST; steered by FP32 and
+// to be steered again
+constexpr int HJ_LARGE = 1, HJ_TURN = 2, HJ_ABOVE = 4, HJ_AGAIN = 8;
 
 // The sweep after one that met a cosine above this is steered in FP32 (46 us in place of 75 us at order 97).  Below it the
 // products that FP32 leaves count: at 1e-3 most Grams took a sweep more (order 97: 550 us, 521 us at 2e-2, 554 us unsteered;
@@ -198,7 +212,9 @@ __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, 
         large = ag * ag > hj_last<T>() * hj_last<T>() * ab;
     }
     if (on && above && (sizeof(T) == 4 || fabsf(u) > 1e-30f)) {
-        if (large) big = 1;
+        if (large || (sizeof(T) == 8 && !STEER && fabsf(u) > hj_turn<T>())) big |= HJ_LARGE;
+        if (sizeof(T) == 4 && fabsf(u) > hj_turn<T>()) big |= HJ_TURN;
+        if (sizeof(T) == 4 && ag * ag > HJ_REST * HJ_REST * ab) big |= HJ_ABOVE;
         T ud, s;
         if constexpr (sizeof(T) == 8) {
             ud = hj_to_double(u);
@@ -668,7 +684,7 @@ __global__ void __launch_bounds__(SH::NT, 1)
     bool steer = sizeof(T) == 8;
     for (int sweep = 0; sweep < max_sweeps && rc > 1; ++sweep) {
         ++nsweeps;
-        int big = 0;   // a rotation that is not small
+        int big = 0;   // HJ_* of this thread's rotations
         for (int blk = 0; blk < 2; ++blk) {   // exact squared norms
             T s = T(0);
             if (grp < b) {
@@ -741,9 +757,14 @@ __global__ void __launch_bounds__(SH::NT, 1)
                 }
                 __syncthreads();
             }
-            if (round == 2 * Ce - 2) {   // did this sweep rotate by more than a little? told to every CTA
-                const int any = __syncthreads_or(big);
-                const int tell = sizeof(T) == 8 && steer ? (any ? 3 : 1) : any;   // a steered sweep is never the last one
+            if (round == 2 * Ce - 2) {   // what this sweep met, told to every CTA
+                int tell = __syncthreads_or(big & HJ_LARGE) ? HJ_LARGE : 0;
+                if constexpr (sizeof(T) == 4) {
+                    if (__syncthreads_or(big & HJ_TURN)) tell |= HJ_TURN;
+                    if (__syncthreads_or(big & HJ_ABOVE)) tell |= HJ_ABOVE;
+                } else if (steer) {
+                    tell = tell ? HJ_LARGE | HJ_AGAIN : HJ_LARGE;   // a steered sweep is never the last one
+                }
                 if (tid < C && crank < Ce) cluster.map_shared_rank(&s_flags[sweep & 1][0], tid)[crank] = tell;
             }
             if (Ce == 1) {
@@ -773,8 +794,8 @@ __global__ void __launch_bounds__(SH::NT, 1)
         }
         int fl = 0;
         for (int r = 0; r < Ce; ++r) fl |= s_flags[sweep & 1][r];
-        if (!fl) break;   // no rotation, or only small ones
-        steer = steer && (fl & 2);
+        if (!(fl & HJ_LARGE) && (fl & (HJ_TURN | HJ_ABOVE)) != (HJ_TURN | HJ_ABOVE)) break;
+        steer = steer && (fl & HJ_AGAIN);
     }
     // ---- 3. eigenvalues (exact squared norms) to CTA 0, decreasing order, truncation rule, normalised kept columns.
     // 2 Ce - 1 moves bring every block home, so player k is where the Cholesky put it.
