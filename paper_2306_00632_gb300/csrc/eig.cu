@@ -48,9 +48,12 @@ __host__ __device__ constexpr double jacobi_tau() { return sizeof(T) == 8 ? 1e-1
 // one-sided Jacobi (FP32): a pair is orthogonal once |a_p . a_q| <= HJ_TAU |a_p| |a_q|.  The normalised columns
 // are then eigenvectors orthonormal to about HJ_TAU; the FP32 dot product itself resolves about 4e-7 at 128 rows.
 constexpr float HJ_TAU = 2e-6f;
-// a sweep whose rotations all had |a_p . a_q| <= HJ_TAU_LAST |a_p| |a_q| is the last one: cyclic Jacobi converges
-// quadratically, so the sweep after it would only meet products near HJ_TAU_LAST^2 ~ HJ_TAU
+// a sweep whose rotations all had |a_p . a_q| <= HJ_TAU_LAST |a_p| |a_q| and turned by a sine of at most HJ_TURN is the last
+// one: a rotation gives the product of two columns at most its sine times another product, so cosines up to
+// HJ_TAU_LAST HJ_TURN = 9e-6 may stay.  (Columns of nearly equal norm turn by up to 45 degrees at any cosine; ended by the
+// cosines alone, the vectors of triples of singular values 1e-4 apart were orthonormal to 4e-4.)
 constexpr float HJ_TAU_LAST = 1.5e-3f;
+constexpr float HJ_TURN = 6e-3f;
 
 // Energy of the Gram outside the Rayleigh-Ritz subspace (trace(G) minus the Ritz values; 0 when the
 // eigensolver's input is the Gram itself).  The FP32 rule (trace minus kept) counts it implicitly.
@@ -581,8 +584,7 @@ __global__ void __launch_bounds__(EIG_THREADS) jacobi_eig_v_kernel(RoundPlan* pl
 //     gamma = a_p . a_q rotates when gamma^2 > tau^2 alpha beta: zeta = (beta - alpha) / (2 gamma),
 //     t = sign(zeta) / (|zeta| + sqrt(1 + zeta^2)), a_p <- c a_p - s a_q, a_q <- s a_p + c a_q, and the
 //     norms follow as alpha - t gamma, beta + t gamma (recomputed exactly at every sweep start).  Sweeps end
-//     when none rotates, or after a sweep whose rotations were all below HJ_TAU_LAST (quadratic convergence
-//     leaves the next sweep's products near HJ_TAU).
+//     when none rotates, or after a sweep whose rotations were all below HJ_TAU_LAST and HJ_TURN.
 //  3. The columns are the players of a round-robin tournament (circle method, one fixed player) on 8 NWA
 //     players, NWA in {2, 4, 8, 16} the fewest warps whose ring holds the rc columns of L: four pair slots per
 //     warp, every lane holding four rows of each of its warp's eight columns in registers.  A step computes
@@ -785,7 +787,7 @@ __global__ void __launch_bounds__(HJ_THREADS) hestenes_eig_kernel(RoundPlan* pla
                     s = c * t;
                     tg = t * gm;
                     rot = 1;
-                    if (gm * gm > taul2 * al * be) big = 1;
+                    if (gm * gm > taul2 * al * be || fabsf(s) > HJ_TURN) big = 1;
                 }
 #pragma unroll
                 for (int j = 0; j < HJ_SLOTS; ++j) {
@@ -859,7 +861,7 @@ __global__ void __launch_bounds__(HJ_THREADS) hestenes_eig_kernel(RoundPlan* pla
             buf ^= 1;
         }
         if (!__syncthreads_or(rot)) break;
-        if (!__syncthreads_or(big)) break;   // only small rotations this sweep: converged to about HJ_TAU
+        if (!__syncthreads_or(big)) break;   // only small rotations this sweep
     }
     // ---- 3. eigenvalues (exact squared norms), decreasing order, truncation rule, normalised kept columns
     __syncthreads();

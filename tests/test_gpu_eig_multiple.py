@@ -69,3 +69,10 @@ def test_f64(api, n, k, gap, draws):
 @pytest.mark.parametrize("n,k,draws", [(9, 9, 60), (32, 24, 40), (97, 48, 20), (128, 72, 12)])
 def test_f32(api, n, k, gap, draws):
     assert _worst(api, n, k, gap, 1, draws, 1e-3) <= 1e-5 + 2 * k * 2.0 ** -24
+
+
+@pytest.mark.parametrize("gap", [1e-2, 1e-4, 1e-6])
+@pytest.mark.parametrize("n,k,draws", [(130, 24, 40), (160, 48, 20), (160, 96, 12)])
+def test_f32_large_contexts(api, n, k, gap, draws):
+    """Contexts above n = 128, whose FP32 Grams and Ritz matrices have an eigensolver of their own (tau 2e-6)."""
+    assert _worst(api, n, k, gap, 1, draws, 1e-3) <= 1.2e-5 + 2 * k * 2.0 ** -24
