@@ -576,10 +576,10 @@ __global__ void __launch_bounds__(SH::NT, 1)
         if (warp == 0) {
             const double d = lane < NQ && dg[lane] > T(0) ? (double)dg[lane] : 0.0;
             const double t = hj_warp_sum(d);
-            if (lane == 0) cluster.map_shared_rank(&s_red[0], 0)[crank] = t;
+            if (lane < C) cluster.map_shared_rank(&s_red[0], lane)[crank] = t;
         }
         cluster.sync();   // columns complete, remote reads done
-        if (crank == 0 && tid == 0) {
+        if (tid == 0) {
             double t = 0.0;
             for (int r = 0; r < C; ++r) t += s_red[r];
             s_rem = t * unscale;
@@ -676,8 +676,14 @@ __global__ void __launch_bounds__(SH::NT, 1)
     }
     if constexpr (sizeof(T) == 8) cluster.sync();   // read by everybody before the blocks move
     else __syncthreads();
-    const T skip = sizeof(T) == 8 && !p.strict ? (T)(1e-3 * bus * (double)__fdividef(1.f, (float)M)) : T(0);
-    // (a direction of discarded energy below budget / (M + 1) in all is discarded with any basis of it)
+    // FP64, plain rule: pairs whose squared norms are both below 1e-3 budget / M are left as they are, since all such columns
+    // together are discarded, in any basis of them.  Not so where the energy outside the columns takes the budget by itself
+    // (a budget below the Gram's rounding, a poor Ritz basis): then nothing is discarded, and what is kept is made orthogonal.
+    T skip = T(0);
+    if constexpr (sizeof(T) == 8) {
+        const double outside = s_rem + (p.rr ? fmax(trace - s_tr, 0.0) + 4e-16 * (double)M * trace : 0.0);
+        if (!p.strict && outside < 0.5 * budget) skip = 1e-3 * bus * (double)__fdividef(1.f, (float)M);
+    }
     const T floor_g = sizeof(T) == 8 ? T(0) : T(1e-12f) * tr;   // FP32 products below this are noise of the factor
     auto column = [&](int set, int blk, int pos) -> T* { return cols + ((set * 2 + blk) * BMAX + pos) * LD; };
     T x[RPL], y[RPL];
