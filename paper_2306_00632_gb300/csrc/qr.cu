@@ -141,18 +141,19 @@ __global__ void __launch_bounds__(32 * SH::NW, 1)
         sig = qr_warp_sum(sig);
         al = __shfl_sync(0xffffffffu, al, j & 31);
         T s2 = fma(al, al, sig), sc = T(1), unsc = T(1);
-        const bool any = !(sig == T(0));   // (a NaN goes on through the column)
-        if (any && s2 < (sizeof(T) == 8 ? T(1e-280) : T(1e-30f))) {   // squares near the end of the range: scaled column
+        if (s2 < (sizeof(T) == 8 ? T(1e-280) : T(1e-30f))) {   // squares near or below the end of the range: scaled column
             sc = sizeof(T) == 8 ? T(0x1p500) : T(0x1p60f);
             unsc = sizeof(T) == 8 ? T(0x1p-500) : T(0x1p-60f);
             sig = T(0);
 #pragma unroll
             for (int q = 0; q < RPL; ++q)
                 if (lane + 32 * q > j) sig = fma(x[q] * sc, x[q] * sc, sig);
+            sig = qr_warp_sum(sig);
             al *= sc;
-            s2 = fma(al, al, qr_warp_sum(sig));
+            s2 = fma(al, al, sig);
         }
-        T nrm = T(0), f = T(0), vj = T(0), beta = al;
+        const bool any = !(sig == T(0));   // (a NaN goes on through the column)
+        T nrm = T(0), f = T(0), vj = T(0), beta = al * unsc;
         if (any) {
             qr_scalars(s2, (T)fabs(al), nrm, f);
             vj = al >= T(0) ? al + nrm : al - nrm;
