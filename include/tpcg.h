@@ -360,6 +360,11 @@ void tpcg_elast_destroy(tpcg_elast e);
  *   correction update of x) take the resolved rule whenever their tolerance is below 1e-8 and the context holds
  *   3 rank_cap columns; 0 one Gram pass with the plain rule. */
 #define TPCG_OPT_RESOLVED 10
+/*   TPCG_OPT_CLUSTER: the most CTAs of a thread-block cluster: 16 (default) where the device grants clusters of 16
+ *   (asked when a context is created), else, and with 8, the portable 8 that every device grants: FP64 Grams above
+ *   order 64 then run on 8 CTAs, the QR of factors with more than 128 (FP64) or 256 (FP32) rows on one, and the
+ *   scalar products of small contexts as six launches.  Read when a kernel is launched or captured. */
+#define TPCG_OPT_CLUSTER 11
 int tpcg_set_option(int key, long long value);
 
 /* Best exponential sum s_R(lambda) = sum_j omega_j exp(-alpha_j lambda) for 1/lambda on [1, M] in the maximum

@@ -24,13 +24,13 @@
 // one CTA's registers with a barrier a step took 0.43 ms.
 #include <math.h>
 
-#include <mutex>
 #include <string>
 #include <type_traits>
 
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "device.cuh"
 #include "eig.cuh"
 
 namespace tpcg {
@@ -943,10 +943,9 @@ __global__ void __launch_bounds__(SH::NT, 1)
 
 namespace {
 template <typename SH>
-int hj_prepare_one() {
+int hj_prepare_one(bool* wide) {
     TPCG_CUDA(cudaFuncSetAttribute(hj_eig_kernel<SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::SMEM));
-    if (SH::C > 8) TPCG_CUDA(cudaFuncSetAttribute(hj_eig_kernel<SH>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    return TPCG_OK;
+    return allow_cluster(hj_eig_kernel<SH>, SH::C, SH::NT, SH::SMEM, wide);
 }
 
 template <typename SH>
@@ -977,23 +976,22 @@ using Hj64a = HjShape<double, 4, 32, 1, 4>;
 using Hj64b = HjShape<double, 8, 32, 2, 4>;
 using Hj64c = HjShape<double, 16, 32, 4, 4>;
 using Hj64d = HjShape<double, 16, 32, 8, 8>;
+// where the device has no clusters of 16
+using Hj64c8 = HjShape<double, 8, 32, 4, 4>;
+using Hj64d8 = HjShape<double, 8, 32, 8, 8>;
+PerDevice hj_device;
 }  // namespace
 
-int hj_prepare() {   // once per device: takes driver locks, so it stays off the launch path
-    static std::mutex mu;
-    static bool done[64] = {};
-    int dev = 0;
-    TPCG_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) dev = 63;
-    std::lock_guard<std::mutex> lock(mu);
-    if (done[dev]) return TPCG_OK;
-    TPCG_TRY(hj_prepare_one<Hj32>());
-    TPCG_TRY(hj_prepare_one<Hj64a>());
-    TPCG_TRY(hj_prepare_one<Hj64b>());
-    TPCG_TRY(hj_prepare_one<Hj64c>());
-    TPCG_TRY(hj_prepare_one<Hj64d>());
-    done[dev] = true;
-    return TPCG_OK;
+int hj_prepare() {
+    return hj_device.prepare([](bool* wide) {
+        TPCG_TRY(hj_prepare_one<Hj32>(wide));
+        TPCG_TRY(hj_prepare_one<Hj64a>(wide));
+        TPCG_TRY(hj_prepare_one<Hj64b>(wide));
+        TPCG_TRY(hj_prepare_one<Hj64c>(wide));
+        TPCG_TRY(hj_prepare_one<Hj64d>(wide));
+        TPCG_TRY(hj_prepare_one<Hj64c8>(wide));
+        return hj_prepare_one<Hj64d8>(wide);
+    });
 }
 
 template <typename T>
@@ -1003,6 +1001,10 @@ int launch_hj(RoundPlan* plan, const T* G, T* S, double* evals, int m, int n, cu
     } else {
         if (n <= Hj64a::ROWS) return hj_launch_one<Hj64a>(plan, G, S, evals, m, st);
         if (n <= Hj64b::ROWS) return hj_launch_one<Hj64b>(plan, G, S, evals, m, st);
+        if (!hj_device.wide()) {
+            if (n <= Hj64c8::ROWS) return hj_launch_one<Hj64c8>(plan, G, S, evals, m, st);
+            return hj_launch_one<Hj64d8>(plan, G, S, evals, m, st);
+        }
         if (n <= Hj64c::ROWS) return hj_launch_one<Hj64c>(plan, G, S, evals, m, st);
         return hj_launch_one<Hj64d>(plan, G, S, evals, m, st);
     }

@@ -21,9 +21,11 @@ int round_resolved(tpcg_ctx c, const tucker_t* y, tucker_t* out, double eps, con
                    double* norm2_slot, tucker_t* E, tucker_t* F, cudaStream_t st);
 int round_mixed(tpcg_ctx c64, tpcg_ctx c32, tucker_t* y64, tucker_t* out32, double eps, const double* eps_dev, int cap,
                 double abs_tol, double* info_dev, cudaStream_t st);
-// Householder QR Y_t = Q_t R_t of the modes with k_t < n (qr.cu), n <= QR_MAXN; W: n x n working copies, ld n everywhere
+// Householder QR Y_t = Q_t R_t of the modes with k_t < n (qr.cu), where qr_fits (n <= QR_MAXN; above 256 in FP32, 128 in FP64
+// only with clusters of 16 CTAs); W: n x n working copies, ld n everywhere
 constexpr int QR_MAXN = 512;
 int qr_prepare();
+bool qr_fits(int n, int elt);
 int dot_prepare();
 template <typename T>
 int launch_qr(const RoundPlan* plan, int n, const T* const* Y, T* const* W, T* const* R, T* const* Q, cudaStream_t st);

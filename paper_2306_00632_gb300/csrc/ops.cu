@@ -9,6 +9,7 @@
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "device.cuh"
 #include "gemm.cuh"
 #include "kernels.cuh"
 
@@ -506,18 +507,12 @@ __global__ void __launch_bounds__(DS_T)
     }
 }
 
-int dot_prepare() {   // clusters above 8 CTAs, once per device (takes driver locks: off the launch path)
-    static std::mutex mu;
-    static bool done[64] = {};
-    int dev = 0;
-    TPCG_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) dev = 63;
-    std::lock_guard<std::mutex> lock(mu);
-    if (done[dev]) return TPCG_OK;
-    TPCG_CUDA(cudaFuncSetAttribute(dot_small_kernel<double>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    TPCG_CUDA(cudaFuncSetAttribute(dot_small_kernel<float>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    done[dev] = true;
-    return TPCG_OK;
+static PerDevice dot_device;
+int dot_prepare() {
+    return dot_device.prepare([](bool* wide) {
+        TPCG_TRY(allow_cluster(dot_small_kernel<double>, DS_C, DS_T, 0, wide));
+        return allow_cluster(dot_small_kernel<float>, DS_C, DS_T, 0, wide);
+    });
 }
 
 template <typename T>
@@ -550,7 +545,7 @@ int dot_impl(tpcg_ctx c, const tucker_t* x, const tucker_t* y, double* out_dev, 
     T* Ta = static_cast<T*>(c->dotT);
     T* Tb = Ta + (long long)rc * rc * rc;
     prof_begin(PK_DOT, st);
-    if (rc <= DS_R) {
+    if (rc <= DS_R && dot_device.wide()) {
         TPCG_TRY(launch_dot_small<T>(x, y, n, rc, out_dev, st));
         prof_end(PK_DOT, st);
         return TPCG_OK;

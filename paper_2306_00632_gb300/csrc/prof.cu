@@ -146,6 +146,8 @@ static std::atomic<int> g_round_rule{-1};
 int round_rule() { return g_round_rule.load(std::memory_order_relaxed); }
 static std::atomic<int> g_resolved{1};
 int resolved_kind() { return g_resolved.load(std::memory_order_relaxed); }
+static std::atomic<int> g_cluster{16};
+int cluster_limit() { return g_cluster.load(std::memory_order_relaxed); }
 }  // namespace tpcg
 
 extern "C" int tpcg_set_option(int key, long long value) {
@@ -187,6 +189,10 @@ extern "C" int tpcg_set_option(int key, long long value) {
     }
     if (key == TPCG_OPT_GRAM_MIN_K && value >= 0 && value <= (1 << 24)) {
         tpcg::g_gram_min_k.store((int)value);
+        return TPCG_OK;
+    }
+    if (key == TPCG_OPT_CLUSTER && (value == 8 || value == 16)) {
+        tpcg::g_cluster.store((int)value);
         return TPCG_OK;
     }
     tpcg::set_error("tpcg_set_option: unknown key or value out of range");

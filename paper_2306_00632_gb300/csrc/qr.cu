@@ -13,11 +13,10 @@
 // Reflectors are kept unscaled, H = I - f v v^T with v = a -+ |a| e_1 and f = 1 / (|a| (|a| + |a_1|)).
 #include <math.h>
 
-#include <mutex>
-
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "device.cuh"
 #include "kernels.cuh"
 
 namespace tpcg {
@@ -287,10 +286,9 @@ __global__ void __launch_bounds__(32 * SH::NW, 1)
 
 namespace {
 template <typename SH>
-int qr_prepare_one() {
+int qr_prepare_one(bool* wide) {
     TPCG_CUDA(cudaFuncSetAttribute(qr_hh_kernel<SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::SMEM));
-    if (SH::C > 8) TPCG_CUDA(cudaFuncSetAttribute(qr_hh_kernel<SH>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    return TPCG_OK;
+    return allow_cluster(qr_hh_kernel<SH>, SH::C, 32 * SH::NW, SH::SMEM, wide);
 }
 
 template <typename SH>
@@ -322,26 +320,25 @@ using Qr64b = QrShape<double, 8, 4, 2, 2, true>;
 using Qr64c = QrShape<double, 8, 8, 4, 2, true>;
 using Qr64d = QrShape<double, 16, 8, 8, 2, false>;
 using Qr64e = QrShape<double, 16, 16, 16, 2, false>;
+PerDevice qr_device;
 }  // namespace
 
-int qr_prepare() {   // once per device: takes driver locks, so it stays off the launch path
-    static std::mutex mu;
-    static bool done[64] = {};
-    int dev = 0;
-    TPCG_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) dev = 63;
-    std::lock_guard<std::mutex> lock(mu);
-    if (done[dev]) return TPCG_OK;
-    TPCG_TRY(qr_prepare_one<Qr32a>());
-    TPCG_TRY(qr_prepare_one<Qr32b>());
-    TPCG_TRY(qr_prepare_one<Qr32c>());
-    TPCG_TRY(qr_prepare_one<Qr64a>());
-    TPCG_TRY(qr_prepare_one<Qr64b>());
-    TPCG_TRY(qr_prepare_one<Qr64c>());
-    TPCG_TRY(qr_prepare_one<Qr64d>());
-    TPCG_TRY(qr_prepare_one<Qr64e>());
-    done[dev] = true;
-    return TPCG_OK;
+int qr_prepare() {
+    return qr_device.prepare([](bool* wide) {
+        TPCG_TRY(qr_prepare_one<Qr32a>(wide));
+        TPCG_TRY(qr_prepare_one<Qr32b>(wide));
+        TPCG_TRY(qr_prepare_one<Qr32c>(wide));
+        TPCG_TRY(qr_prepare_one<Qr64a>(wide));
+        TPCG_TRY(qr_prepare_one<Qr64b>(wide));
+        TPCG_TRY(qr_prepare_one<Qr64c>(wide));
+        TPCG_TRY(qr_prepare_one<Qr64d>(wide));
+        return qr_prepare_one<Qr64e>(wide);
+    });
+}
+
+bool qr_fits(int n, int elt) {
+    const int narrow = elt == 4 ? Qr32b::ROWS : Qr64c::ROWS;   // the largest on clusters of 8
+    return n <= narrow || (n <= QR_MAXN && qr_device.wide());
 }
 
 template <typename T>

@@ -232,7 +232,7 @@ __device__ void householder_qr(const T* Y, T* A, T* R, T* Q, int rows, int k, lo
     }
 }
 
-// Alg. 1 step 1 above n = QR_MAXN: Y_t = Q_t R_t for the modes with k_t < n, one CTA per mode (n x k_t, ld n)
+// Alg. 1 step 1 where qr.cu does not fit: Y_t = Q_t R_t for the modes with k_t < n, one CTA per mode (n x k_t, ld n)
 template <typename T>
 __global__ void __launch_bounds__(1024) qr_kernel(const RoundPlan* __restrict__ plan, const T* Y0, const T* Y1,
                                                   const T* Y2, T* W0, T* W1, T* W2, T* R0, T* R1, T* R2, T* Q0,
@@ -639,7 +639,7 @@ int round_stage12(tpcg_ctx c, tucker_t* y, double eps, const double* eps_dev, in
     TPCG_CHECK_LAUNCH();
     // step 1: QR where k_t < n
     prof_begin(PK_QR, st);
-    if (n <= QR_MAXN) {
+    if (qr_fits(n, (int)sizeof(T))) {
         const T* Y[3];
         T *W[3], *R[3], *Q[3];
         for (int t = 0; t < 3; ++t) {
