@@ -310,9 +310,10 @@ void tpcg_elast_destroy(tpcg_elast e);
 
 /* ------------------------------------------------------------------------------------ tuning */
 /* Launch-shape options (no counterpart in the paper), process-wide:
- *   TPCG_OPT_GEMM_CTAS_PER_SM: CTA budget per SM of the grouped GEMM launches (0 = one CTA per output tile
- *   and argument group; 1..64 caps the grid and the kernel strides over the groups; default 2, measured best
- *   with 32 solves at once: 4.0 against 3.6 solves/s uncapped). */
+ *   TPCG_OPT_GEMM_CTAS_PER_SM: CTA budget per SM of the grouped GEMM launches, in CTAs of 256 threads (those of 128
+ *   threads, which the FP64 and most of the FP32 contractions have, count half): 1..64 caps the grid and the CTAs
+ *   stride over the output tiles, 0 launches one CTA per tile of the worst case; default 2, measured best with 32
+ *   solves at once.  The tensor-core contractions (TPCG_OPT_TC) have grids of their own. */
 #define TPCG_OPT_GEMM_CTAS_PER_SM 1
 /*   TPCG_OPT_EXPSUM_BEST: which exponential sums (Prop. 1) tpcg_setup / tpcg_elast_setup build for the FD
  *   preconditioner: 1 (default) the best sums of tpcg_expsum_best, whose R_P reproduces Table 1; 0 the

@@ -200,8 +200,9 @@ __global__ void __launch_bounds__(G64_NT, 4) gemm64_kernel(const GemmArgs* __res
 int launch_gemm64(const GemmArgs* args, const int* count_dev, int ngroups, int bmax, int Mmax, int Nmax, bool ta, bool tb,
                   cudaStream_t st) {
     const long long tiles = (long long)((Mmax + G64_T - 1) / G64_T) * ((Nmax + G64_T - 1) / G64_T) * ngroups * bmax;
-    // four CTAs an SM: one is enough for the FP64 units, the others hide the loads of a K-step
-    const int grid = (int)std::min<long long>(tiles * G64_PART, 4LL * sm_count());
+    // four CTAs an SM by default: one is enough for the FP64 units, the others hide the loads of a K-step
+    const int per_sm = 2 * gemm_ctas_per_sm();   // (the budget counts CTAs of 256 threads)
+    const int grid = (int)std::min<long long>(tiles * G64_PART, per_sm > 0 ? (long long)per_sm * sm_count() : 65535LL);
     gemm64_kernel<<<grid, G64_NT, 0, st>>>(args, count_dev, ngroups, ta, tb, sm_count());
     TPCG_CHECK_LAUNCH();
     return TPCG_OK;
