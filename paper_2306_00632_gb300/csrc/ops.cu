@@ -545,7 +545,8 @@ int dot_impl(tpcg_ctx c, const tucker_t* x, const tucker_t* y, double* out_dev, 
     T* Ta = static_cast<T*>(c->dotT);
     T* Tb = Ta + (long long)rc * rc * rc;
     prof_begin(PK_DOT, st);
-    if (rc <= DS_R && dot_device.wide()) {
+    // (TPCG_OPT_TC 1 asks for the FP32 contractions on the tensor cores, which the single launch has none of)
+    if (rc <= DS_R && dot_device.wide() && !(sizeof(T) == 4 && tc_kind() == 1)) {
         TPCG_TRY(launch_dot_small<T>(x, y, n, rc, out_dev, st));
         prof_end(PK_DOT, st);
         return TPCG_OK;

@@ -2,6 +2,7 @@
 import pytest
 
 import synth
+from oracle import tucker
 from tests.graph_helpers import kernels
 
 pytestmark = pytest.mark.gpu
@@ -39,3 +40,22 @@ def test_ctas_per_sm_reaches_both_types(mods, dtype, name):
         assert largest() > 3 * sms * 256
     finally:
         api.set_option(lib.OPT_GEMM_CTAS_PER_SM, 2)
+
+
+def test_tensor_cores_reach_small_scalar_products(mods):
+    api, lib = mods
+    n = 24
+    X = synth.random_tucker((n, n, n), (5, 6, 7), seed=5)
+    Y = synth.random_tucker((n, n, n), (8, 3, 4), seed=6)
+    try:
+        api.set_option(lib.OPT_TC, 1)
+        for dtype in (0, 1):
+            x, y = (api.Tucker.from_numpy(T[0], T[1], dtype=dtype) for T in (X, Y))
+            ctx = api.Ctx(n, n, 16, dtype=dtype)
+            out = torch.zeros(1, dtype=torch.float64, device="cuda")
+            names = [k for k, *_ in kernels(lambda: api.tucker_dot(ctx, x, y, out=out))]
+            assert any("gemm_tc" in k for k in names) == (dtype == 1), names
+            # 22 bits of each operand over the sums of five contractions
+            assert abs(api.tucker_dot(ctx, x, y).item() - tucker.dot(X, Y)) <= 1e-5 * tucker.norm(X) * tucker.norm(Y)
+    finally:
+        api.set_option(lib.OPT_TC, 0)
