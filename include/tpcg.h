@@ -328,7 +328,8 @@ void tpcg_elast_destroy(tpcg_elast e);
 /*   TPCG_OPT_DST: how the preconditioner applies the sine block U_dft of App. B (Alg. 4): 1 (default) for n1 <= 256 and
  *   like ends two half-size dense products (its columns are even or odd about the middle), else batched FFTs,
  *   O(n1 log n1) per column, by Bluestein's chirp-z identity for any n1 <= 1024 (power-of-two FFTs of size
- *   >= 2 n1 - 1 in shared memory); 0 the dense n1 x n1 product with the stored sine matrix. */
+ *   >= 2 n1 - 1 in shared memory); 2 the FFTs for every n1 <= 1024; 0 the dense n1 x n1 product with the stored
+ *   sine matrix. */
 #define TPCG_OPT_DST 4
 /*   TPCG_OPT_TC: where the FP32 contractions (Alg. 1 Z formation, mode Grams, projections and factor updates, the
  *   scalar products) run: 1 on the tensor cores (tcgen05, 3xTF32 products with FP32 accumulation in tensor

@@ -93,7 +93,7 @@ int chirp_tables(int n1, int p, int k0, int k1, ChirpInfo* info, std::vector<dou
 template <typename T>
 int launch_chirp(tpcg_problem pb, int kind, const TuckerDesc* sd, int mult, int rp_guard, int vcap, int maxcols,
                  const T* const* X, T* const* Y, int ldx, int ldy, cudaStream_t st);
-int dst_kind();   // TPCG_OPT_DST: 1 half matrices or FFTs, 0 dense sine matrix
+int dst_kind();   // TPCG_OPT_DST: 1 half matrices or FFTs, 2 FFTs, 0 dense sine matrix
 // Alg. 4 with the two half matrices of a symmetric sine block (fd_fold.cu), for n1 up to FD_FOLD_MAX
 constexpr int FD_FOLD_MAX = 256;
 bool fd_fold_fits(tpcg_problem pb);

@@ -867,7 +867,7 @@ int fd_impl(tpcg_problem pb, tpcg_ctx c, const tucker_t* s, tucker_t* v, cudaStr
                                         static_cast<T*>(v->U[0]), static_cast<T*>(v->U[1]),
                                         static_cast<T*>(v->U[2]), ga, counts, v->cap, err);
     TPCG_CHECK_LAUNCH();
-    const bool fft = pb->d_chirp != nullptr && dst_kind() == 1;
+    const bool fft = pb->d_chirp != nullptr && dst_kind() != 0;
     const T* fx[3] = {buf[0][0], buf[1][0], buf[2][0]};
     T* fy[3] = {buf[0][1], buf[1][1], buf[2][1]};
     if (fft)   // u_t = U_dft^T T_t by FFTs

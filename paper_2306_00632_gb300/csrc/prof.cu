@@ -163,7 +163,7 @@ extern "C" int tpcg_set_option(int key, long long value) {
         tpcg::g_eig_kind.store((int)value);
         return TPCG_OK;
     }
-    if (key == TPCG_OPT_DST && (value == 0 || value == 1)) {
+    if (key == TPCG_OPT_DST && value >= 0 && value <= 2) {
         tpcg::g_dst_kind.store((int)value);
         return TPCG_OK;
     }
