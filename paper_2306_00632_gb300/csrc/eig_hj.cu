@@ -32,6 +32,7 @@
 #include "common.cuh"
 #include "device.cuh"
 #include "eig.cuh"
+#include "recip.cuh"
 
 namespace tpcg {
 
@@ -45,7 +46,7 @@ namespace cgx = cooperative_groups;
 // most its largest cosine times its largest sine.  It is the last one when its cosines were all below `last` and its
 // |u| = |tan(theta / 2)| all below `turn`: 2 turn last = 2e-14 (FP64) and 9e-6 (FP32) may stay.  The cosines alone say
 // nothing where norms nearly coincide: there a cosine of 1e-10 turns by 45 degrees (with that rule the kept vectors of triples of
-// singular values 1e-9 apart were orthonormal to 2e-10 in place of 1e-14, in FP32 to 4e-4).  FP32: wide turns do not
+// singular values 1e-9 apart were orthonormal to 2e-10 in place of 1e-14, in FP32 to 4e-4; the flags cost the FP32 step 2.5%).  FP32: wide turns do not
 // count in a sweep whose cosines were all below `rest`, which may stay; pairs of equal norm would go on turning on
 // the rounding of their products.
 template <typename T>
@@ -82,28 +83,6 @@ struct HjShape {
 __device__ __forceinline__ double hj_warp_sum(double v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
-}
-
-// An SM issues an FP64 instruction of a warp every 64 cycles and quarter, conversions included, so what only steers
-// the iteration is done in FP32 and conversions by moving bits.
-// v 2^-off as a float (mantissa cut, not rounded; 0 below FP32's range), and a normal float as a double times 2^off
-__device__ __forceinline__ float hj_to_float(double v, int off) {
-    const int hi = __double2hiint(v);
-    const int e = ((hi >> 20) & 0x7ff) - (1023 - 127) - off;
-    const int bits = (hi & 0x80000000) | (e << 23) | ((hi & 0xfffff) << 3) | ((unsigned)__double2loint(v) >> 29);
-    return e > 0 ? __int_as_float(bits) : 0.f;
-}
-__device__ __forceinline__ double hj_to_double(float f, int off = 0) {
-    const unsigned b = __float_as_uint(f);
-    const int hi = (int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + ((unsigned)(1023 - 127 + off) << 20)));
-    return __hiloint2double(hi, (int)(b << 29));
-}
-
-// 1 / sqrt(d) for d in FP32's normal range: an FP32 estimate and one third-order correction (relative error a few ulp)
-__device__ __forceinline__ double hj_rsqrt(double d) {
-    const double y = hj_to_double(rsqrtf(hj_to_float(d, 0)));
-    const double e = fma(-(d * y), y, 1.0);
-    return fma(y * e, fma(e, 0.375, 0.5), y);
 }
 
 // This lane's rows of a column at a: rows gl + LPP q, the first rpl of them; in FP32 with a warp per pair the four rows
@@ -163,11 +142,11 @@ __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, 
     if constexpr (STEER) {
 #pragma unroll
         for (int q = 0; q < RPL; ++q)
-            if (q < rpl) g0 = fmaf(hj_to_float(x[q], 0), hj_to_float(y[q], 0), g0);
+            if (q < rpl) g0 = fmaf(bits_to_float(x[q]), bits_to_float(y[q]), g0);
 #pragma unroll
         for (int o = LPP / 2; o > 0; o >>= 1) g0 += __shfl_xor_sync(0xffffffffu, g0, o);
-        a0 = hj_to_float(ax, 0);
-        b0 = hj_to_float(ay, 0);
+        a0 = bits_to_float(ax);
+        b0 = bits_to_float(ay);
         const float sc = __int_as_float(0x7f000000 - (__float_as_int(fmaxf(a0, b0)) & 0x7f800000));   // larger norm to [1, 2)
         fa = a0 * sc;
         fb = b0 * sc;
@@ -178,10 +157,10 @@ __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, 
     } else if constexpr (sizeof(T) == 8) {   // by a power of two near the larger norm: nothing that counts leaves FP32's range
         const int hx = __double2hiint(ax), hy = __double2hiint(ay), hs = __double2hiint(skip);
         off = (max(hx, hy) >> 20) - 1023;
-        fa = hj_to_float(ax, off);
-        fb = hj_to_float(ay, off);
-        fg = hj_to_float(g, off);
-        fd = hj_to_float(ay - ax, off);
+        fa = bits_to_float(ax, off);
+        fb = bits_to_float(ay, off);
+        fg = bits_to_float(g, off);
+        fd = bits_to_float(ay - ax, off);
         on = hx > hs || hy > hs;      // both far below the budget: all discarded, whatever their products
     } else {
         fa = ax;
@@ -217,20 +196,18 @@ __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, 
         if (sizeof(T) == 4 && ag * ag > HJ_REST * HJ_REST * ab) big |= HJ_ABOVE;
         T ud, s;
         if constexpr (sizeof(T) == 8) {
-            ud = hj_to_double(u);
-            const double u2 = hj_to_double(2.f * u);
+            ud = bits_to_double(u);
+            const double u2 = bits_to_double(2.f * u);
             if (fabsf(u) < 1e-4f && fabsf(u) > 1e-15f) {   // 2 u (1 - u^2) to u^4
-                s = fma(-u2, hj_to_double(u * u), u2);
+                s = fma(-u2, bits_to_double(u * u), u2);
             } else {
                 const float qf = fmaf(u, u, 1.f);
-                const double q = fma(ud, ud, 1.0), r0 = hj_to_double(__fdividef(1.f, qf));
-                const double e = fma(-q, r0, 1.0);
-                s = u2 * fma(r0, fma(e, e, e), r0);
+                s = u2 * recip_from(fma(ud, ud, 1.0), bits_to_double(__fdividef(1.f, qf)));
             }
         } else {
             ud = u;
-            const float q = fmaf(u, u, 1.f), r0 = __fdividef(1.f, q);
-            s = 2.f * u * fmaf(r0, fmaf(-q, r0, 1.f), r0);
+            const float q = fmaf(u, u, 1.f);
+            s = 2.f * u * recip_from(q, __fdividef(1.f, q));
         }
         if constexpr (hj_vec<T, LPP, RPL>) {
             const float2 mu = make_float2(-u, -u), s2 = make_float2(s, s);
@@ -254,11 +231,11 @@ __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, 
         }
         const float tg = t * fg;   // the norms are exact again at the next sweep
         if constexpr (STEER) {
-            ax = hj_to_double(fmaxf(a0 - t * g0, 0.f));
-            ay = hj_to_double(fmaxf(b0 + t * g0, 0.f));
+            ax = bits_to_double(fmaxf(a0 - t * g0, 0.f));
+            ay = bits_to_double(fmaxf(b0 + t * g0, 0.f));
         } else if constexpr (sizeof(T) == 8) {
             if (fabsf(tg) > 1e-30f) {
-                const double v = hj_to_double(tg, off);
+                const double v = bits_to_double(tg, off);
                 ax -= v;
                 ay += v;
             }
@@ -426,7 +403,7 @@ __global__ void __launch_bounds__(SH::NT, 1)
             const int key = hi > noise ? hi : -1;
             const int best = __reduce_max_sync(FULL, key);
             const int piv = __ffs(__ballot_sync(FULL, key == best)) - 1;
-            float left = hi > 0 ? hj_to_float(d, 0) : 0.f;
+            float left = hi > 0 ? bits_to_float(d) : 0.f;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) left += __shfl_xor_sync(FULL, left, o);
             if (best < 0 || !(left > stop_rem)) break;   // the same in every thread of the cluster
@@ -441,8 +418,7 @@ __global__ void __launch_bounds__(SH::NT, 1)
             }
             // A -= a a^T / d of the column a as it is; the scaling of L's column waits until it is read back
             const double dp = __shfl_sync(FULL, d, piv);
-            const double r0 = hj_to_double(__fdividef(1.f, hj_to_float(dp, 0)));
-            const double er = fma(-dp, r0, 1.0), invd = fma(r0, fma(er, er, er), r0);
+            const double invd = recip_mid(dp);
             gone |= 1u << piv;
             if (tid == 0) {
                 piv_of[k] = (short)piv;
@@ -513,7 +489,7 @@ __global__ void __launch_bounds__(SH::NT, 1)
                 }
             } else if (warp == 1) {   // what is left of the trace
                 const double d = lane < NQ ? dg[lane] : -1.0;
-                float left = __double2hiint(d) > 0 ? hj_to_float(d, 0) : 0.f;
+                float left = __double2hiint(d) > 0 ? bits_to_float(d) : 0.f;
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) left += __shfl_xor_sync(FULL, left, o);
                 if (lane < C) cluster.map_shared_rank(&s_left[par][0], lane)[crank] = left;
@@ -535,8 +511,7 @@ __global__ void __launch_bounds__(SH::NT, 1)
 #pragma unroll
             for (int a = 0; a < RT; ++a) col[a] = alive[a] ? src[row + a * NT] : T(0);
             const double d = s_piv[par][own];
-            const double r0 = hj_to_double(__fdividef(1.f, hj_to_float(d, 0)));
-            const double er = fma(-d, r0, 1.0), invd = fma(r0, fma(er, er, er), r0);
+            const double invd = recip_mid(d);
             T* lk = lbuf[par];
             T* out = k % C == crank ? cols + (k / C) * LD : nullptr;   // (a store to global memory here makes the barrier wait)
 #pragma unroll
@@ -622,8 +597,7 @@ __global__ void __launch_bounds__(SH::NT, 1)
             if (warp == piv % NW) {
                 // l = A[:, piv] / sqrt(d), zero on the rows of earlier pivots.  (An IEEE square root and divisions here kept
                 // the other warps waiting for 1000 of 2500 cycles a step.)
-                const float d = __int_as_float(best), y0 = rsqrtf(d);
-                const float inv = fmaf(y0 * fmaf(-d * y0, y0, 1.f), 0.5f, y0);
+                const float d = __int_as_float(best), inv = rsqrt_from(d, rsqrtf(d));
                 const int ap = piv / NW;
                 float* out = k % C == crank ? S + (long long)k * n : nullptr;
 #pragma unroll
@@ -668,7 +642,7 @@ __global__ void __launch_bounds__(SH::NT, 1)
         const int i = e % ROWS, slot = e / ROWS, k = slot * Ce + crank;
         T v = T(0);
         if constexpr (sizeof(T) == 8) {   // from where the Cholesky left it, scaled by the pivot (kept by every CTA)
-            if (k < rc) v = cluster.map_shared_rank(cols, k % C)[(k / C) * LD + i] * hj_rsqrt(lam[k]);
+            if (k < rc) v = cluster.map_shared_rank(cols, k % C)[(k / C) * LD + i] * rsqrt(lam[k]);
         } else {
             if (k < rc && i < M) v = S[i + (long long)k * n];
         }
@@ -889,7 +863,7 @@ __global__ void __launch_bounds__(SH::NT, 1)
     for (int blk = 0; blk < 2; ++blk) {
         const int k = (2 * grp + blk) * Ce + crank;
         if (grp < b && k < rc && ord[k] < s && lam[k] > 0.0) {
-            const T inv = lam[k] > 1e-30 ? (T)hj_rsqrt(lam[k]) : (T)(1.0 / sqrt(lam[k]));
+            const T inv = (T)rsqrt(lam[k]);
             const T* a = column(set, blk, grp);
             for (int i = gl; i < M; i += LPP) S[i + (long long)ord[k] * n] = a[i] * inv;
         }

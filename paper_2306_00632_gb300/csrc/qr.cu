@@ -7,7 +7,7 @@
 //
 // What bounds it: k steps of one warp's chain (update of column j + 1, its norm, the reflector, the barrier), about 0.6 us in
 // FP32 and, at 64 cycles an FP64 instruction, 2 us in FP64.  Measured at n = 128 and 106 / 60 / 30 columns, three modes: FP32
-// 111 / 60 / 33 us on four CTAs of 16 warps (one CTA of 32 warps 158 / 81 / 36, eight of 16 98 / 57 / 32); FP64 453 / 222 / 112 us
+// 111 / 60 / 33 us on four CTAs of 16 warps (one CTA of 32 warps 158 / 81 / 36, eight of 16 98 / 57 / 32); FP64 445 / 222 / 111 us
 // on eight CTAs of 8 warps (eight of 4 532 / 259 / 111, sixteen of 4 435 / 223 / 113).  The kernel this replaces, one CTA with
 // its working copy in global memory, took 400 us in FP32 at 106 columns and 190 us in FP64 for 17 columns at n = 32 (now 41).
 // Reflectors are kept unscaled, H = I - f v v^T with v = a -+ |a| e_1 and f = 1 / (|a| (|a| + |a_1|)).
@@ -22,32 +22,6 @@
 namespace tpcg {
 
 namespace cgx = cooperative_groups;
-
-// 1 / sqrt(d) of any normal positive d: an FP32 estimate on the mantissa and a third-order correction (a few ulp; the
-// library's FP64 square root and division are 40 dependent FP64 instructions)
-__device__ __forceinline__ double qr_rsqrt(double d) {
-    const int e = (((__double2hiint(d) >> 20) & 0x7ff) - 1023) & ~1;
-    const double m = __hiloint2double(__double2hiint(d) - (e << 20), __double2loint(d));   // in [1, 4)
-    const double y = (double)rsqrtf((float)m);
-    const double r = fma(-(m * y), y, 1.0);
-    const double z = fma(y * r, fma(r, 0.375, 0.5), y);
-    return __hiloint2double(__double2hiint(z) - ((e / 2) << 20), __double2loint(z));
-}
-
-// |a| and f of a reflector from s2 = |a|^2 > 0 and a1 = |a_1|
-__device__ __forceinline__ void qr_scalars(double s2, double a1, double& nrm, double& f) {
-    const double r = qr_rsqrt(s2);
-    nrm = s2 * r;
-    // 1 / (|a| + |a_1|): |a| <= that <= 2 |a|, so times r it is in [1, 2]
-    const double d = fma(a1, r, 1.0);
-    const double y = (double)(1.f / (float)d);
-    const double e = fma(-d, y, 1.0);
-    f = r * r * fma(y, fma(e, e, e), y);
-}
-__device__ __forceinline__ void qr_scalars(float s2, float a1, float& nrm, float& f) {
-    nrm = sqrtf(s2);
-    f = 1.f / (nrm * (nrm + a1));
-}
 
 template <typename T>
 __device__ __forceinline__ T qr_warp_sum(T v) {
@@ -154,7 +128,8 @@ __global__ void __launch_bounds__(32 * SH::NW, 1)
         const bool any = !(sig == T(0));   // (a NaN goes on through the column)
         T nrm = T(0), f = T(0), vj = T(0), beta = al * unsc;
         if (any) {
-            qr_scalars(s2, (T)fabs(al), nrm, f);
+            nrm = sqrt(s2);
+            f = T(1) / (nrm * (nrm + fabs(al)));
             vj = al >= T(0) ? al + nrm : al - nrm;
             beta = (al >= T(0) ? -nrm : nrm) * unsc;
         }
