@@ -8,7 +8,7 @@
 //  2. Plane rotations from the right make the columns of L orthogonal, L J = U Sigma: the normalised columns are
 //     eigenvectors of G and their squared norms its eigenvalues, and no rotation matrix is accumulated.
 //  3. The columns lie in shared memory in 2 Ce blocks of b, two blocks per CTA of the cluster.  In a round every CTA
-//     rotates all b^2 pairs of one column of each of its blocks, b disjoint pairs at a time (16 lanes to a pair; the
+//     rotates all b^2 pairs of one column of each of its blocks, b disjoint pairs at a time (a warp to a pair; the
 //     top block's columns stay in registers), then the blocks move by the circle method through distributed shared
 //     memory.  2 Ce - 1 rounds and the pairs inside the blocks make a sweep in which every pair meets once.  The
 //     cluster waits for itself once a round, not once a step.
@@ -46,9 +46,9 @@ namespace cgx = cooperative_groups;
 // most its largest cosine times its largest sine.  It is the last one when its cosines were all below `last` and its
 // |u| = |tan(theta / 2)| all below `turn`: 2 turn last = 2e-14 (FP64) and 9e-6 (FP32) may stay.  The cosines alone say
 // nothing where norms nearly coincide: there a cosine of 1e-10 turns by 45 degrees (with that rule the kept vectors of triples of
-// singular values 1e-9 apart were orthonormal to 2e-10 in place of 1e-14, in FP32 to 4e-4; the flags cost the FP32 step 2.5%).  FP32: wide turns do not
-// count in a sweep whose cosines were all below `rest`, which may stay; pairs of equal norm would go on turning on
-// the rounding of their products.
+// singular values 1e-9 apart were orthonormal to 2e-10 in place of 1e-14, in FP32 to 4e-4; the flags cost the FP32 step 2.5%).
+// FP32: wide turns do not count in a sweep whose cosines were all below `rest`, which may stay; pairs of equal norm would
+// go on turning on the rounding of their products.
 template <typename T>
 __host__ __device__ constexpr T hj_tau() { return sizeof(T) == 8 ? T(1e-14) : T(5e-7); }
 template <typename T>
@@ -66,18 +66,17 @@ constexpr int HJ_LARGE = 1, HJ_TURN = 2, HJ_ABOVE = 4, HJ_AGAIN = 8;
 // order 32 188 us, 187 us and 213 us; three Grams of order 64 in a sum 703, 690 and 779 us).
 constexpr float HJ_STEER = 2e-2f;
 
-// Shape of a launch: C CTAs, LPP lanes per pair of columns, RPL rows per lane (orders up to LPP RPL), BT pairs a CTA
-// takes at a time before another CTA joins.
-template <typename T_, int C_, int LPP_, int RPL_, int BT_>
+// Shape of a launch: C CTAs, a warp to a pair of columns, RPL rows a lane (orders up to 32 RPL), BT pairs a CTA takes at a
+// time before another CTA joins.
+template <typename T_, int C_, int RPL_, int BT_>
 struct HjShape {
     using T = T_;
-    static constexpr int C = C_, LPP = LPP_, RPL = RPL_, BT = BT_;
-    static constexpr int ROWS = LPP * RPL;
+    static constexpr int C = C_, RPL = RPL_, BT = BT_;
+    static constexpr int ROWS = 32 * RPL;
     static constexpr int BMAX = (ROWS / C + 1) / 2;              // columns of the largest block, pairs at once
-    static constexpr int NT = BMAX * LPP > 128 ? BMAX * LPP : 128;
-    static constexpr int LD = sizeof(T) == 4 && LPP < 32 ? ROWS + LPP : ROWS;   // FP32: a warp's columns on different banks
+    static constexpr int NT = BMAX * 32 > 128 ? BMAX * 32 : 128;
     // two sets of two blocks of columns; the Cholesky's own columns lie in the second set
-    static constexpr size_t SMEM = (size_t)4 * BMAX * LD * sizeof(T);
+    static constexpr size_t SMEM = (size_t)4 * BMAX * ROWS * sizeof(T);
 };
 
 __device__ __forceinline__ double hj_warp_sum(double v) {
@@ -85,44 +84,43 @@ __device__ __forceinline__ double hj_warp_sum(double v) {
     return v;
 }
 
-// This lane's rows of a column at a: rows gl + LPP q, the first rpl of them; in FP32 with a warp per pair the four rows
-// 4 gl + q in one 16-byte access (all of them: rows past the order are zero, and an FP32 FMA is cheaper than a test)
-template <typename T, int LPP, int RPL>
-constexpr bool hj_vec = sizeof(T) == 4 && LPP == 32 && RPL == 4;
-template <typename T, int LPP, int RPL>
-__device__ __forceinline__ void hj_load(T (&x)[RPL], const T* a, int gl, int rpl) {
-    if constexpr (hj_vec<T, LPP, RPL>) {
-        const float4 v = *reinterpret_cast<const float4*>(a + 4 * gl);
+// This lane's rows of a column at a: rows lane + 32 q, the first rpl of them; in FP32 the four rows 4 lane + q in one 16-byte
+// access (all of them: rows past the order are zero, and an FP32 FMA is cheaper than a test)
+template <typename T, int RPL>
+constexpr bool hj_vec = sizeof(T) == 4 && RPL == 4;
+template <typename T, int RPL>
+__device__ __forceinline__ void hj_load(T (&x)[RPL], const T* a, int lane, int rpl) {
+    if constexpr (hj_vec<T, RPL>) {
+        const float4 v = *reinterpret_cast<const float4*>(a + 4 * lane);
         x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
     } else {
 #pragma unroll
         for (int q = 0; q < RPL; ++q)
-            if (q < rpl) x[q] = a[gl + LPP * q];
+            if (q < rpl) x[q] = a[lane + 32 * q];
     }
 }
-template <typename T, int LPP, int RPL>
-__device__ __forceinline__ void hj_save(const T (&x)[RPL], T* a, int gl, int rpl) {
-    if constexpr (hj_vec<T, LPP, RPL>) {
-        *reinterpret_cast<float4*>(a + 4 * gl) = make_float4(x[0], x[1], x[2], x[3]);
+template <typename T, int RPL>
+__device__ __forceinline__ void hj_save(const T (&x)[RPL], T* a, int lane, int rpl) {
+    if constexpr (hj_vec<T, RPL>) {
+        *reinterpret_cast<float4*>(a + 4 * lane) = make_float4(x[0], x[1], x[2], x[3]);
     } else {
 #pragma unroll
         for (int q = 0; q < RPL; ++q)
-            if (q < rpl) a[gl + LPP * q] = x[q];
+            if (q < rpl) a[lane + 32 * q] = x[q];
     }
 }
 
-// One pair: x and y are this lane's rows of the two columns (zero for an idle group), ax and ay their squared norms.
-// Whole warps call it.  A pair with |x . y| above tau |x| |y| is rotated: u = tan(theta / 2), s = sin(theta), applied
-// as the shears x -= u y, y += s x, x -= u y (three FMAs an element).  The angle needs no more than FP32: an error of
-// 1e-6 in it leaves 1e-6 of the product for the next sweep; s = 2 u / (1 + u^2) has the working precision, so that the
-// shears make an orthogonal matrix.
+// One pair, by a whole warp: x and y are this lane's rows of the two columns, ax and ay their squared norms.  A pair with
+// |x . y| above tau |x| |y| is rotated: u = tan(theta / 2), s = sin(theta), applied as the shears x -= u y, y += s x,
+// x -= u y (three FMAs an element).  The angle needs no more than FP32: an error of 1e-6 in it leaves 1e-6 of the product
+// for the next sweep; s = 2 u / (1 + u^2) has the working precision, so that the shears make an orthogonal matrix.
 //
 // STEER (FP64, the first sweeps): everything but the shears and s in FP32 as well, the dot product and the norms included.
 // Their error of 1e-6 |x| |y| stays for the sweeps that follow, and an FP64 step of 17 instructions at 32 rows becomes one of 8.
-template <typename T, int LPP, int RPL, bool STEER = false>
+template <typename T, int RPL, bool STEER = false>
 __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, int rpl, T skip, T floor_g, int& big) {
     T g = T(0);
-    if constexpr (hj_vec<T, LPP, RPL>) {
+    if constexpr (hj_vec<T, RPL>) {
         const float2 g2 = __ffma2_rn(make_float2(x[2], x[3]), make_float2(y[2], y[3]),
                                      __fmul2_rn(make_float2(x[0], x[1]), make_float2(y[0], y[1])));
         g = g2.x + g2.y;
@@ -133,7 +131,7 @@ __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, 
     }
     if constexpr (!STEER) {
 #pragma unroll
-        for (int o = LPP / 2; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+        for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
     }
     float fa, fb, fg, fd;   // |x|^2, |y|^2, x . y, |y|^2 - |x|^2
     int off = 0;
@@ -144,7 +142,7 @@ __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, 
         for (int q = 0; q < RPL; ++q)
             if (q < rpl) g0 = fmaf(bits_to_float(x[q]), bits_to_float(y[q]), g0);
 #pragma unroll
-        for (int o = LPP / 2; o > 0; o >>= 1) g0 += __shfl_xor_sync(0xffffffffu, g0, o);
+        for (int o = 16; o > 0; o >>= 1) g0 += __shfl_xor_sync(0xffffffffu, g0, o);
         a0 = bits_to_float(ax);
         b0 = bits_to_float(ay);
         const float sc = __int_as_float(0x7f000000 - (__float_as_int(fmaxf(a0, b0)) & 0x7f800000));   // larger norm to [1, 2)
@@ -209,7 +207,7 @@ __device__ __forceinline__ void hj_pair(T (&x)[RPL], T (&y)[RPL], T& ax, T& ay, 
             const float q = fmaf(u, u, 1.f);
             s = 2.f * u * recip_from(q, __fdividef(1.f, q));
         }
-        if constexpr (hj_vec<T, LPP, RPL>) {
+        if constexpr (hj_vec<T, RPL>) {
             const float2 mu = make_float2(-u, -u), s2 = make_float2(s, s);
 #pragma unroll
             for (int q = 0; q < 4; q += 2) {
@@ -295,11 +293,10 @@ __global__ void __launch_bounds__(SH::NT, 1)
     hj_eig_kernel(RoundPlan* plan, const typename SH::T* __restrict__ G, typename SH::T* __restrict__ S, double* evals,
                   int m, int max_sweeps, double* prof) {
     using T = typename SH::T;
-    constexpr int C = SH::C, LPP = SH::LPP, RPL = SH::RPL, LD = SH::LD, ROWS = SH::ROWS, BMAX = SH::BMAX, NT = SH::NT;
+    constexpr int C = SH::C, RPL = SH::RPL, ROWS = SH::ROWS, LD = ROWS, BMAX = SH::BMAX, NT = SH::NT;
     constexpr int NQ = 2 * BMAX;                    // columns of G per CTA (Cholesky)
     constexpr unsigned FULL = 0xffffffffu;
     static_assert(NQ <= 32, "one lane per column in the search for the pivot");
-    static_assert(LPP == 32, "a warp per pair: no warp holds a pair beside an idle one");
     cgx::cluster_group cluster = cgx::this_cluster();
     const int crank = (int)cluster.block_rank();
     RoundPlan& p = *plan;
@@ -376,7 +373,7 @@ __global__ void __launch_bounds__(SH::NT, 1)
     const double unscale = __hiloint2double((1023 - s_exp) << 20, 0);
     const double bus = s_bus;   // the budget on that scale
     const T tr = s_trs;
-    const int rpl = (M + LPP - 1) / LPP;
+    const int rpl = (M + 31) / 32;
     // ---- 1. pivoted Cholesky.  How the columns of L are spread over the cluster depends on their number: they wait in
     // shared memory (FP64) or in S (FP32)
     int rc = 0;
@@ -636,7 +633,6 @@ __global__ void __launch_bounds__(SH::NT, 1)
     // (k / Ce) & 1, position k / (2 Ce).  The others only wait with the cluster.
     const int Ce = max(1, min(C, (rc + 2 * SH::BT - 1) / (2 * SH::BT)));
     const int b = crank < Ce ? max(1, ((rc + Ce - 1) / Ce + 1) / 2) : 0;
-    const int grp = tid / LPP, gl = tid % LPP;
     int set = sizeof(T) == 8 ? 1 : 0, nsweeps = 0;
     for (int e = tid; e < 2 * b * ROWS; e += NT) {
         const int i = e % ROWS, slot = e / ROWS, k = slot * Ce + crank;
@@ -667,22 +663,22 @@ __global__ void __launch_bounds__(SH::NT, 1)
         int big = 0;   // HJ_* of this thread's rotations
         for (int blk = 0; blk < 2; ++blk) {   // exact squared norms
             T s = T(0);
-            if (grp < b) {
-                hj_load<T, LPP, RPL>(x, column(set, blk, grp), gl, rpl);
+            if (warp < b) {
+                hj_load<T, RPL>(x, column(set, blk, warp), lane, rpl);
 #pragma unroll
                 for (int q = 0; q < RPL; ++q)
-                    if (q < rpl || hj_vec<T, LPP, RPL>) s = fma(x[q], x[q], s);
+                    if (q < rpl || hj_vec<T, RPL>) s = fma(x[q], x[q], s);
             }
 #pragma unroll
-            for (int o = LPP / 2; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
-            if (grp < b && gl == 0) nrm[set][blk][grp] = s;
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
+            if (warp < b && lane == 0) nrm[set][blk][warp] = s;
         }
         __syncthreads();
         // pairs inside the two blocks (round robin on b rounded up to even players)
         const int be = (b + 1) & ~1;
         for (int step = 0; step < be - 1; ++step) {
             const int half = be / 2;
-            const int blk = grp / half, k = grp - blk * half;
+            const int blk = warp / half, k = warp - blk * half;
             int i = -1, j = -1;
             if (blk < 2) {
                 const int P = be - 1;
@@ -694,46 +690,40 @@ __global__ void __launch_bounds__(SH::NT, 1)
                 if (i > j) { const int t = i; i = j; j = t; }
                 if (j >= b) i = -1;
             }
-            const bool on = i >= 0;
-            if (__any_sync(FULL, on)) {
-                T* xp = column(set, on ? blk : 0, on ? i : 0);
-                T* yp = column(set, on ? blk : 0, on ? j : 0);
-                T ax = on ? nrm[set][blk][i] : T(0), ay = on ? nrm[set][blk][j] : T(0);
-                hj_load<T, LPP, RPL>(x, xp, gl, rpl);
-                hj_load<T, LPP, RPL>(y, yp, gl, rpl);
-                if (sizeof(T) == 8 && steer) hj_pair<T, LPP, RPL, sizeof(T) == 8>(x, y, ax, ay, rpl, skip, floor_g, big);
-                else hj_pair<T, LPP, RPL>(x, y, ax, ay, rpl, skip, floor_g, big);
-                if (on) {
-                    hj_save<T, LPP, RPL>(x, xp, gl, rpl);
-                    hj_save<T, LPP, RPL>(y, yp, gl, rpl);
-                    if (gl == 0) { nrm[set][blk][i] = ax; nrm[set][blk][j] = ay; }
-                }
+            if (i >= 0) {
+                T* xp = column(set, blk, i);
+                T* yp = column(set, blk, j);
+                T ax = nrm[set][blk][i], ay = nrm[set][blk][j];
+                hj_load<T, RPL>(x, xp, lane, rpl);
+                hj_load<T, RPL>(y, yp, lane, rpl);
+                if (sizeof(T) == 8 && steer) hj_pair<T, RPL, sizeof(T) == 8>(x, y, ax, ay, rpl, skip, floor_g, big);
+                else hj_pair<T, RPL>(x, y, ax, ay, rpl, skip, floor_g, big);
+                hj_save<T, RPL>(x, xp, lane, rpl);
+                hj_save<T, RPL>(y, yp, lane, rpl);
+                if (lane == 0) { nrm[set][blk][i] = ax; nrm[set][blk][j] = ay; }
             }
             __syncthreads();
         }
         for (int round = 0; round < 2 * Ce - 1; ++round) {
-            const bool act = grp < b;   // (b is 0 where the CTA has no columns; a warp with no pair at all skips the steps)
-            const bool wact = LPP == 32 ? act : warp * (32 / LPP) < b;
+            const bool act = warp < b;   // (b is 0 where the CTA has no columns)
             T ax = T(0);
-            if (wact) {
-                hj_load<T, LPP, RPL>(x, column(set, 0, act ? grp : 0), gl, rpl);
-                ax = act ? nrm[set][0][grp] : T(0);
+            if (act) {
+                hj_load<T, RPL>(x, column(set, 0, warp), lane, rpl);
+                ax = nrm[set][0][warp];
             }
-            int j = grp;
-            T* yp = column(set, 1, act ? grp : 0);
+            int j = warp;
+            T* yp = column(set, 1, act ? warp : 0);
             for (int k = 0; k < b; ++k) {
-                if (wact) {
-                    T ay = act ? nrm[set][1][j] : T(0);
-                    hj_load<T, LPP, RPL>(y, yp, gl, rpl);
-                    if (sizeof(T) == 8 && steer) hj_pair<T, LPP, RPL, sizeof(T) == 8>(x, y, ax, ay, rpl, skip, floor_g, big);
-                    else hj_pair<T, LPP, RPL>(x, y, ax, ay, rpl, skip, floor_g, big);
-                    if (act) {
-                        hj_save<T, LPP, RPL>(y, yp, gl, rpl);
-                        if (gl == 0) nrm[set][1][j] = ay;
-                        ++j;
-                        yp += LD;
-                        if (j == b) { j = 0; yp -= b * LD; }
-                    }
+                if (act) {
+                    T ay = nrm[set][1][j];
+                    hj_load<T, RPL>(y, yp, lane, rpl);
+                    if (sizeof(T) == 8 && steer) hj_pair<T, RPL, sizeof(T) == 8>(x, y, ax, ay, rpl, skip, floor_g, big);
+                    else hj_pair<T, RPL>(x, y, ax, ay, rpl, skip, floor_g, big);
+                    hj_save<T, RPL>(y, yp, lane, rpl);
+                    if (lane == 0) nrm[set][1][j] = ay;
+                    ++j;
+                    yp += LD;
+                    if (j == b) { j = 0; yp -= b * LD; }
                 }
                 __syncthreads();
             }
@@ -749,8 +739,8 @@ __global__ void __launch_bounds__(SH::NT, 1)
             }
             if (Ce == 1) {
                 if (act) {
-                    hj_save<T, LPP, RPL>(x, column(set, 0, grp), gl, rpl);
-                    if (gl == 0) nrm[set][0][grp] = ax;
+                    hj_save<T, RPL>(x, column(set, 0, warp), lane, rpl);
+                    if (lane == 0) nrm[set][0][warp] = ax;
                 }
                 cluster.sync();
                 continue;
@@ -761,13 +751,13 @@ __global__ void __launch_bounds__(SH::NT, 1)
             const int tb = crank == 0 ? 0 : (crank == Ce - 1 ? 1 : 0);
             const int bc = crank == 0 ? 1 : crank - 1, bb = crank == 0 ? 0 : 1;
             if (act) {
-                hj_save<T, LPP, RPL>(x, cluster.map_shared_rank(cols, tc) + ((ns * 2 + tb) * BMAX + grp) * LD, gl, rpl);
-                if (gl == 0) {
-                    cluster.map_shared_rank(&nrm[0][0][0], tc)[(ns * 2 + tb) * BMAX + grp] = ax;
-                    cluster.map_shared_rank(&nrm[0][0][0], bc)[(ns * 2 + bb) * BMAX + grp] = nrm[set][1][grp];
+                hj_save<T, RPL>(x, cluster.map_shared_rank(cols, tc) + ((ns * 2 + tb) * BMAX + warp) * LD, lane, rpl);
+                if (lane == 0) {
+                    cluster.map_shared_rank(&nrm[0][0][0], tc)[(ns * 2 + tb) * BMAX + warp] = ax;
+                    cluster.map_shared_rank(&nrm[0][0][0], bc)[(ns * 2 + bb) * BMAX + warp] = nrm[set][1][warp];
                 }
-                hj_load<T, LPP, RPL>(y, column(set, 1, grp), gl, rpl);
-                hj_save<T, LPP, RPL>(y, cluster.map_shared_rank(cols, bc) + ((ns * 2 + bb) * BMAX + grp) * LD, gl, rpl);
+                hj_load<T, RPL>(y, column(set, 1, warp), lane, rpl);
+                hj_save<T, RPL>(y, cluster.map_shared_rank(cols, bc) + ((ns * 2 + bb) * BMAX + warp) * LD, lane, rpl);
             }
             cluster.sync();
             set = ns;
@@ -781,16 +771,16 @@ __global__ void __launch_bounds__(SH::NT, 1)
     // 2 Ce - 1 moves bring every block home, so player k is where the Cholesky put it.
     for (int blk = 0; blk < 2; ++blk) {
         T s = T(0);
-        if (grp < b) {
-            hj_load<T, LPP, RPL>(x, column(set, blk, grp), gl, rpl);
+        if (warp < b) {
+            hj_load<T, RPL>(x, column(set, blk, warp), lane, rpl);
 #pragma unroll
             for (int q = 0; q < RPL; ++q)
-                if (q < rpl || hj_vec<T, LPP, RPL>) s = fma(x[q], x[q], s);
+                if (q < rpl || hj_vec<T, RPL>) s = fma(x[q], x[q], s);
         }
 #pragma unroll
-        for (int o = LPP / 2; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
-        const int k = (2 * grp + blk) * Ce + crank;
-        if (grp < b && gl == 0 && k < rc)
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
+        const int k = (2 * warp + blk) * Ce + crank;
+        if (warp < b && lane == 0 && k < rc)
             for (int r = 0; r < C; ++r) cluster.map_shared_rank(lam, r)[k] = (double)s;
     }
     cluster.sync();
@@ -861,11 +851,11 @@ __global__ void __launch_bounds__(SH::NT, 1)
     cluster.sync();
     const int s = s_keep;
     for (int blk = 0; blk < 2; ++blk) {
-        const int k = (2 * grp + blk) * Ce + crank;
-        if (grp < b && k < rc && ord[k] < s && lam[k] > 0.0) {
+        const int k = (2 * warp + blk) * Ce + crank;
+        if (warp < b && k < rc && ord[k] < s && lam[k] > 0.0) {
             const T inv = (T)rsqrt(lam[k]);
-            const T* a = column(set, blk, grp);
-            for (int i = gl; i < M; i += LPP) S[i + (long long)ord[k] * n] = a[i] * inv;
+            const T* a = column(set, blk, warp);
+            for (int i = lane; i < M; i += 32) S[i + (long long)ord[k] * n] = a[i] * inv;
         }
     }
     if constexpr (sizeof(T) == 8) {
@@ -945,14 +935,14 @@ int hj_launch_one(RoundPlan* plan, const typename SH::T* G, typename SH::T* S, d
 // instead of 12 pairs before another CTA joins within 5%.  FP64: one pair of columns for each quarter of an SM, by the
 // largest order.  More CTAs for the same columns lose to the cluster's barriers (order 32 of 128 possible: 222 us on four,
 // 323 us on sixteen), fewer to the FP64 pipes (order 120: 1.5 ms on sixteen, 2.0 ms on eight).
-using Hj32 = HjShape<float, 4, 32, 4, 12>;
-using Hj64a = HjShape<double, 4, 32, 1, 4>;
-using Hj64b = HjShape<double, 8, 32, 2, 4>;
-using Hj64c = HjShape<double, 16, 32, 4, 4>;
-using Hj64d = HjShape<double, 16, 32, 8, 8>;
+using Hj32 = HjShape<float, 4, 4, 12>;
+using Hj64a = HjShape<double, 4, 1, 4>;
+using Hj64b = HjShape<double, 8, 2, 4>;
+using Hj64c = HjShape<double, 16, 4, 4>;
+using Hj64d = HjShape<double, 16, 8, 8>;
 // where the device has no clusters of 16
-using Hj64c8 = HjShape<double, 8, 32, 4, 4>;
-using Hj64d8 = HjShape<double, 8, 32, 8, 8>;
+using Hj64c8 = HjShape<double, 8, 4, 4>;
+using Hj64d8 = HjShape<double, 8, 8, 8>;
 PerDevice hj_device;
 }  // namespace
 
