@@ -20,9 +20,9 @@
 #include <math.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "common.cuh"
+#include "device.cuh"
 #include "gemm.cuh"
 #include "kernels.cuh"
 
@@ -353,18 +353,12 @@ static int fd_fold_prepare_one() {
     return TPCG_OK;
 }
 
-int fd_fold_prepare() {   // once per device: takes driver locks, so it stays off the launch path
-    static std::mutex mu;
-    static bool done[64] = {};
-    int dev = 0;
-    TPCG_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) dev = 63;
-    std::lock_guard<std::mutex> lock(mu);
-    if (done[dev]) return TPCG_OK;
-    TPCG_TRY(fd_fold_prepare_one<double>());
-    TPCG_TRY(fd_fold_prepare_one<float>());
-    done[dev] = true;
-    return TPCG_OK;
+int fd_fold_prepare() {
+    static PerDevice device;
+    return device.prepare([](bool*) {
+        TPCG_TRY(fd_fold_prepare_one<double>());
+        return fd_fold_prepare_one<float>();
+    });
 }
 
 }  // namespace tpcg

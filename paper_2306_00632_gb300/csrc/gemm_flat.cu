@@ -9,9 +9,8 @@
 // 5.3 -> 3.8 ms; a scalar product of rank 6 at n = 32 130 -> 66 us.
 #include <math.h>
 
-#include <mutex>
-
 #include "common.cuh"
+#include "device.cuh"
 #include "gemm.cuh"
 
 namespace tpcg {
@@ -393,21 +392,16 @@ template int launch_gemm32<false, false>(const GemmArgs*, const int*, int, int, 
 template int launch_gemm32<false, true>(const GemmArgs*, const int*, int, int, int, int, bool, cudaStream_t);
 template int launch_gemm32<true, false>(const GemmArgs*, const int*, int, int, int, int, bool, cudaStream_t);
 
-// dynamic shared memory above 48 KB, once per device (takes driver locks: off the launch path)
+// dynamic shared memory above 48 KB
 int gemm32_prepare() {
-    static std::mutex mu;
-    static bool done[64] = {};
-    int dev = 0;
-    TPCG_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) dev = 63;
-    std::lock_guard<std::mutex> lock(mu);
-    if (done[dev]) return TPCG_OK;
-    const int b = (int)G32<128, 128, 8>::SMEM;
-    TPCG_CUDA(cudaFuncSetAttribute(gemm32_kernel<128, 128, 8, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, b));
-    TPCG_CUDA(cudaFuncSetAttribute(gemm32_kernel<128, 128, 8, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, b));
-    TPCG_CUDA(cudaFuncSetAttribute(gemm32_kernel<128, 128, 8, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, b));
-    done[dev] = true;
-    return TPCG_OK;
+    static PerDevice device;
+    return device.prepare([](bool*) {
+        const int b = (int)G32<128, 128, 8>::SMEM;
+        TPCG_CUDA(cudaFuncSetAttribute(gemm32_kernel<128, 128, 8, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, b));
+        TPCG_CUDA(cudaFuncSetAttribute(gemm32_kernel<128, 128, 8, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, b));
+        TPCG_CUDA(cudaFuncSetAttribute(gemm32_kernel<128, 128, 8, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, b));
+        return TPCG_OK;
+    });
 }
 
 }  // namespace tpcg

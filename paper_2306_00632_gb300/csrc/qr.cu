@@ -7,9 +7,10 @@
 //
 // What bounds it: k steps of one warp's chain (update of column j + 1, its norm, the reflector, the barrier), about 0.6 us in
 // FP32 and, at 64 cycles an FP64 instruction, 2 us in FP64.  Measured at n = 128 and 106 / 60 / 30 columns, three modes: FP32
-// 111 / 60 / 33 us on four CTAs of 16 warps (one CTA of 32 warps 158 / 81 / 36, eight of 16 98 / 57 / 32); FP64 445 / 222 / 111 us
-// on eight CTAs of 8 warps (eight of 4 532 / 259 / 111, sixteen of 4 435 / 223 / 113).  The kernel this replaces, one CTA with
-// its working copy in global memory, took 400 us in FP32 at 106 columns and 190 us in FP64 for 17 columns at n = 32 (now 41).
+// 111 / 60 / 33 us on four CTAs of 16 warps (one CTA of 32 warps 158 / 81 / 36, eight of 16 98 / 57 / 32); FP64 445 / 222 /
+// 111 us on eight CTAs of 8 warps (eight of 4 532 / 259 / 111, sixteen of 4 435 / 223 / 113; square root and division are
+// CUDA's: an FP32 estimate and a correction in their place took 447 us).  The kernel this replaces, one CTA with its working
+// copy in global memory, took 400 us in FP32 at 106 columns and 190 us in FP64 for 17 columns at n = 32 (now 41).
 // Reflectors are kept unscaled, H = I - f v v^T with v = a -+ |a| e_1 and f = 1 / (|a| (|a| + |a_1|)).
 #include <math.h>
 
