@@ -282,9 +282,10 @@ def _roofline(prof, dt_name, lib, step_ms_total):
     # (bf16 2250, FP32 75, FP64 1.25 TFLOP/s dense nominal)
     alu = {"f64": bf16 * 1.25 / 2250.0, "f32": bf16 * 75.0 / 2250.0}
     classes = ["zgemm", "zblk", "gram", "eig", "proj", "qr", "apply", "fd"]
-    # DRAM bytes per launch of the FP32 eigensolver from one ncu capture of this workload (dram__bytes_read.sum +
-    # dram__bytes_write.sum, mean of 2 launches of hestenes_eig_kernel); other kernels: no capture, traffic null
-    ncu_traffic = {"eig": 118656.0} if dt_name == "mixed" else {}
+    # DRAM bytes per launch of the FP32 eigensolver (hj_eig_kernel) from one ncu capture of a truncated sum at n = 128
+    # (dram__bytes_read.sum + dram__bytes_write.sum, mean of its 3 launches, Grams of order 128; a solve's are mostly
+    # smaller); other kernels: no capture, traffic null
+    ncu_traffic = {"eig": 134912.0} if dt_name == "mixed" else {}
     dom = max(classes, key=lambda k: prof[k]["ms"])
     d = prof[dom]
     per_launch_ms = d["ms"] / max(d["launches"], 1)

@@ -346,9 +346,10 @@ void tpcg_elast_destroy(tpcg_elast e);
  *   partials: less partial traffic and block start-up, which pays when many solves share the device), 0 (default)
  *   always uses the most partials.  Read when a truncation is launched or captured. */
 #define TPCG_OPT_GRAM_MIN_K 7
-/*   TPCG_OPT_GEMM_KIND: the FP32 SIMT contractions: 2 (default) 128 threads per 64 x 64 output tile, 8 x 4 outputs
- *   per thread (16-byte shared loads, 32 FMAs per 3 loads), operands copied by cp.async through three shared
- *   stages; 1 the same tile staged through registers and two stages; 0 256 threads, 4 x 4 outputs per thread. */
+/*   TPCG_OPT_GEMM_KIND: the FP32 SIMT contractions: 2 (default) a flat list of the output tiles of all groups (64 x 64 to
+ *   128 x 128 by the sides' bounds, 8 x 4 or 8 x 8 outputs per thread, paired FMAs), operands copied by cp.async through
+ *   three shared stages; 1 64 x 64 tiles of 128 threads, 8 x 4 outputs each, staged through registers and two stages;
+ *   0 256 threads, 4 x 4 outputs each.  Scalar products of contexts of rank cap at most 32 are one launch of their own. */
 #define TPCG_OPT_GEMM_KIND 8
 /*   TPCG_OPT_ROUND_RULE: the FP64 truncation rule of tucker_round (Alg. 1 step 3 on mode Grams): -1 (default)
  *   automatic, strict below eps = 1e-7 (every discarded Gram eigenvalue charged its rounding uncertainty

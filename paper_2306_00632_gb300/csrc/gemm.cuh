@@ -2,9 +2,12 @@
 // rank-dependent sizes decided on the GPU (truncation ranks) need no host round trip and the launch
 // sequence is fixed (CUDA-graph capturable).  Column-major, op(A) is M x K, op(B) is K x N.
 //
-// Tiling: 64 x 64 output tile per CTA, K-step 16, 256 threads, 4 x 4 outputs per thread held in
-// registers; operands staged through two shared-memory stages (the next K-step is fetched into registers
-// while the current one is consumed), with loads coalesced along the contiguous index.
+// The kernels that run by default are in gemm_flat.cu (a flat list of the output tiles of all groups).  Here: the argument
+// dispatch, and the FP32 kernels of TPCG_OPT_GEMM_KIND 0 and 1, whose grids walk over the groups.
+//
+// Their tiling: 64 x 64 outputs per CTA, K-step 16; kind 0 256 threads with 4 x 4 outputs each in registers, kind 1 128
+// threads with 8 x 4; operands staged through two shared-memory stages (the next K-step is fetched into registers while
+// the current one is consumed), with loads coalesced along the contiguous index.
 #pragma once
 
 #include <algorithm>
